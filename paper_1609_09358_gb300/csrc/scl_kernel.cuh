@@ -12,11 +12,14 @@
 // (metric, index) order -- the paper's pruned pseudo sort d = sum H(m_c - m_j) made a total order
 // by the index tie-break -- and the rank < L candidates survive, renumbered in ascending index.
 //
-// Leaf blocks in registers: the tree below level 6 is a 32-bit leaf block.  Lane p holds path p's
-// LLR arrays of levels 5..1 (62 values) and its partial sums of levels 0..4 (one word each) in
-// registers; the 32 bits of a block are unrolled, so every level index is a compile-time constant.
-// When a list step duplicates paths, a survivor copies from its parent's lane (shuffles) only the
-// leaf levels that a later bit of the block reads before rewriting -- a set known at compile time.
+// Leaf blocks: the tree below level 6 is a 32-bit leaf block.  Lane p holds path p's LLR arrays of
+// levels 4..1 (30 values) and its partial sums of levels 0..4 (one word each) in registers; level 5
+// stays in shared memory, one row per path.  Aligned nodes of 32, 16, 8 and 4 bits that are all
+// frozen or all information are taken whole where that gives the bit-by-bit result exactly
+// (leaf_frozen, leaf_all_hard); the rest goes bit by bit.  When a list step duplicates paths, a
+// survivor copies from its parent's lane (shuffles) only the leaf levels that a later bit of the
+// block reads before rewriting: level k after bit r iff bit k-1 of r is clear, the partial sum of
+// level k iff bit k of r is set.
 //
 // Upper levels (LLR 6..n-1, partial sums 5..n) are touched once per block.  They use lazy copies:
 // every upper level keeps L physical arrays and a path holds one 5-bit pointer per level, packed in
@@ -85,10 +88,8 @@ struct SCLPlan {
 // pad makes both the warp's row-wise writes and the lanes' per-path reads bank-conflict free) and
 // then read into the path's registers.
 constexpr int kSclStage = 33;
-// elements per lane and round of the element-parallel upper-level updates (measured: 8 beats 4,
-// which waits on L2 once per 4 loads, and 16, whose registers cost more than the overlap gains
-// once 16 warps share the SM)
-constexpr int kSclUpRound = 8;
+// units (of four elements) per lane and round of the element-parallel upper-level updates
+constexpr int kSclUpRound = 2;
 __host__ __device__ inline long long scl_smem_llr_words(int KS, int L) { return KS >= 6 ? (long long)L * ((2 << KS) - 64) : 0; }
 __host__ __device__ inline long long scl_smem_c_words(int KC, int L) { return KC >= 5 ? (long long)L * (scl_cssum(KC + 1) - 5) : 0; }
 // `lists` = frames per warp (1, or 2 with half-warp lists): the shared-memory budget of a frame
@@ -108,7 +109,7 @@ __host__ __device__ inline SCLPlan scl_plan(int N, int L, bool all_smem, int lis
         p.KC = 4;
         while (p.KC + 1 <= n && 4 * scl_smem_c_words(p.KC + 1, L) * lists <= 2048) ++p.KC;
     }
-    // per list: [C levels 5..KC][LLR levels 6..KS][level-5 staging, L rows of 33 words]; per warp:
+    // per list: [LLR levels 6..KS][level-5 staging, L rows of 33 words][C levels 5..KC]; per warp:
     // the lists, then 16 words of list-step scratch
     p.list_words = (int)(scl_smem_llr_words(p.KS, L) + scl_smem_c_words(p.KC, L)) + L * kSclStage;
     p.list_words = (p.list_words + 3) & ~3;
@@ -262,27 +263,9 @@ struct SCLWarp {
     }
 };
 
-// ------------------------------------------------------------------ leaf block (compile time)
-__host__ __device__ constexpr int ctz_c(int v)
-{
-    int c = 0;
-    while (!(v & 1)) {
-        v >>= 1;
-        ++c;
-    }
-    return c;
-}
-// Is leaf level k (1..5) read, before being rewritten, by a later bit of the block than r?
-__host__ __device__ constexpr bool leaf_live(int r, int k)
-{
-    for (int q = r + 1; q < 32; ++q) {
-        const int t = ctz_c(q);
-        if (t + 1 == k) return true;
-        if (t >= k) return false;
-    }
-    return false;
-}
-
+// ------------------------------------------------------------------ leaf block
+// A 32-bit leaf block is walked as a tree over the path's registers: level 5 stays in the shared
+// staging rows (a path keeps the number of its row), levels 4..1 live in registers.
 template <int LEN>
 __device__ __forceinline__ void leaf_f(const float (&src)[2 * LEN], float (&dst)[LEN])
 {
@@ -303,106 +286,66 @@ __device__ __forceinline__ void leaf_copy(float (&a)[LEN], int parent)
 }
 
 struct Leaf {
-    float l5[32], l4[16], l3[8], l2[4], l1[2];
+    float l4[16], l3[8], l2[4], l1[2];
     uint32_t c[5];  // partial sums of the left siblings at levels 0..4
+    int row;        // staging row of this path's level 5
 };
 
-// LLR of bit r of the block (levels written: ctz(r)..1, read: ctz(r)+1 and c[ctz(r)])
-template <int R>
-__device__ __forceinline__ float leaf_llr(Leaf& f)
+// Metric of a node whose 2^K leaves are all frozen, from the node's LLRs: every leaf LLR (partial
+// sums 0, so g is a plain addition) in order, each penalty added in order -- the same operations
+// as bit by bit, without the bit loop.  m - min(lambda, 0) = m + |lambda| [lambda < 0].
+template <int LEN>
+__device__ __forceinline__ void leaf_frozen(const float (&a)[LEN], float& pm)
 {
-    if constexpr (R == 0) {
-        leaf_f<16>(f.l5, f.l4);
-        leaf_f<8>(f.l4, f.l3);
-        leaf_f<4>(f.l3, f.l2);
-        leaf_f<2>(f.l2, f.l1);
-        return xmin(f.l1[0], f.l1[1]);
+    if constexpr (LEN == 1) {
+        pm = __fsub_rn(pm, fminf(a[0], 0.0f));
     } else {
-        constexpr int t = ctz_c(R);
-        if constexpr (t == 4) leaf_g<16>(f.l5, f.l4, f.c[4]);
-        if constexpr (t == 3) leaf_g<8>(f.l4, f.l3, f.c[3]);
-        if constexpr (t == 2) leaf_g<4>(f.l3, f.l2, f.c[2]);
-        if constexpr (t == 1) leaf_g<2>(f.l2, f.l1, f.c[1]);
-        if constexpr (t == 0) return scl_g(f.l1[0], f.l1[1], f.c[0] & 1u);
-        if constexpr (t >= 4) leaf_f<8>(f.l4, f.l3);
-        if constexpr (t >= 3) leaf_f<4>(f.l3, f.l2);
-        if constexpr (t >= 2) leaf_f<2>(f.l2, f.l1);
-        return xmin(f.l1[0], f.l1[1]);
-    }
-}
-
-// The partial-sum step with the bit index r at run time (warp-uniform): kc = trailing ones of r
-// levels fold in predicated steps, no jump (measured faster than dispatching leaf_psum<R> by a
-// switch on r; the LLR step keeps the switch, which measured faster than its runtime form).
-__device__ __forceinline__ uint32_t leaf_psum_rt(Leaf& f, uint32_t bitv, int r)
-{
-    if (!(r & 1)) {  // even bits (half of them): the bit itself is the level-0 partial sum
-        f.c[0] = bitv;
-        return bitv;
-    }
-    if (!(r & 2)) {  // bits 1 mod 4 (a quarter): one fold into level 1
-        const uint32_t v1 = ((bitv ^ f.c[0]) & 0x1u) | ((bitv & 0x1u) << 1);
-        f.c[1] = v1;
-        return v1;
-    }
-    const int kc = __ffs(~r) - 1;
-    uint32_t v = bitv;
-    if (kc > 0) v = ((v ^ f.c[0]) & 0x1u) | ((v & 0x1u) << 1);
-    if (kc > 1) v = ((v ^ f.c[1]) & 0x3u) | ((v & 0x3u) << 2);
-    if (kc > 2) v = ((v ^ f.c[2]) & 0xFu) | ((v & 0xFu) << 4);
-    if (kc > 3) v = ((v ^ f.c[3]) & 0xFFu) | ((v & 0xFFu) << 8);
-    if (kc > 4) v = ((v ^ f.c[4]) & 0xFFFFu) | ((v & 0xFFFFu) << 16);
-    if (kc == 0) f.c[0] = v;
-    if (kc == 1) f.c[1] = v;
-    if (kc == 2) f.c[2] = v;
-    if (kc == 3) f.c[3] = v;
-    if (kc == 4) f.c[4] = v;
-    return v;
-}
-
-// after a duplicating list step at bit r: survivors take the live leaf state of their parents
-template <int R>
-__device__ __forceinline__ void leaf_inherit(Leaf& f, int parent)
-{
-    if constexpr (leaf_live(R, 5)) leaf_copy<32>(f.l5, parent);
-    if constexpr (leaf_live(R, 4)) leaf_copy<16>(f.l4, parent);
-    if constexpr (leaf_live(R, 3)) leaf_copy<8>(f.l3, parent);
-    if constexpr (leaf_live(R, 2)) leaf_copy<4>(f.l2, parent);
-    if constexpr (leaf_live(R, 1)) leaf_copy<2>(f.l1, parent);
+        constexpr int H = LEN / 2;
+        float b[H];
 #pragma unroll
-    for (int k = 0; k < 5; ++k) f.c[k] = __shfl_sync(0xffffffffu, f.c[k], parent);
+        for (int j = 0; j < H; ++j) b[j] = xmin(a[j], a[j + H]);
+        leaf_frozen<H>(b, pm);
+#pragma unroll
+        for (int j = 0; j < H; ++j) b[j] = __fadd_rn(a[j + H], a[j]);
+        leaf_frozen<H>(b, pm);
+    }
 }
 
-// The same inheritance with the bit index at run time: `live` = bit k-1 set when leaf level k is
-// live after bit r (leaf_live_mask); one copy of the code serves every bit of the block.
-// Closed form of the same table: level k is next touched at q, the first multiple of 2^(k-1) after
-// r; bit q reads it (by g) iff ctz(q) = k-1, rewrites it iff ctz(q) >= k.
-__host__ __device__ constexpr uint32_t leaf_live_mask(int r)
+// A node of 2^K information bits, decided at once.  Let every path take its hard decisions inside
+// the node: f keeps the smaller magnitude and g then adds magnitudes of equal signs, so the first
+// leaf's |lambda| is m = min |a_j| and no later leaf's is smaller (also after rounding, which is
+// monotone).  So if the full list's largest metric is below every path's metric plus m, the list
+// step's shortcut holds at the first bit and, metrics unchanged, at every later one: the survivors
+// are the paths themselves with the sign bits of a as the node's codeword.  If the condition
+// fails, the first bit's shortcut fails as well.  (A zero LLR makes m = 0 and fails it, so the
+// signs are those of nonzero values.)
+template <int W, int LEN, class Get>
+__device__ __forceinline__ bool leaf_all_hard(const Lanes<W>& sg, Get a, float pm, int act, int L, uint32_t& v)
 {
-    uint32_t m = 0;
-    for (int k = 1; k <= 5; ++k) {
-        const int q = (r | ((1 << (k - 1)) - 1)) + 1;
-        if (q < 32 && ((q >> (k - 1)) & 1)) m |= 1u << (k - 1);
+    if constexpr (W == 32) {
+        if (act != L) return false;
+    } else {
+        if (!__all_sync(0xffffffffu, act == L || act == 0)) return false;
     }
-    return m;
-}
-constexpr bool leaf_live_mask_matches()
-{
-    for (int r = 0; r < 32; ++r)
-        for (int k = 1; k <= 5; ++k)
-            if (((leaf_live_mask(r) >> (k - 1)) & 1u) != (leaf_live(r, k) ? 1u : 0u)) return false;
-    return true;
-}
-static_assert(leaf_live_mask_matches(), "closed form of the leaf liveness table");
-__device__ __forceinline__ void leaf_inherit_rt(Leaf& f, int parent, uint32_t live)
-{
-    if (live & 16u) leaf_copy<32>(f.l5, parent);
-    if (live & 8u) leaf_copy<16>(f.l4, parent);
-    if (live & 4u) leaf_copy<8>(f.l3, parent);
-    if (live & 2u) leaf_copy<4>(f.l2, parent);
-    if (live & 1u) leaf_copy<2>(f.l1, parent);
+    float m[LEN >= 4 ? 4 : LEN];
+    v = 0u;
 #pragma unroll
-    for (int k = 0; k < 5; ++k) f.c[k] = __shfl_sync(0xffffffffu, f.c[k], parent);
+    for (int j = LEN - 1; j >= 0; --j) {
+        const float x = a(j);
+        v = __funnelshift_l(__float_as_uint(x), v, 1);
+        constexpr int Q = LEN >= 4 ? 4 : LEN;
+        m[j % Q] = j + Q >= LEN ? fabsf(x) : fminf(m[j % Q], fabsf(x));
+    }
+    float mm = m[0];
+#pragma unroll
+    for (int q = 1; q < (LEN >= 4 ? 4 : LEN); ++q) mm = fminf(mm, m[q]);
+    const bool on = sg.pl < act;
+    const uint32_t hd_max = sg.red_max(on ? __float_as_uint(pm) : 0u);
+    const uint32_t pen_min = sg.red_min(on ? __float_as_uint(__fadd_rn(pm, mm)) : 0xffffffffu);
+    if constexpr (W == 32)
+        return hd_max < pen_min;
+    else
+        return __all_sync(0xffffffffu, hd_max < pen_min || act == 0);
 }
 
 // Launches the persistent CA-SCL grid (defined in scl_launch.cu).  `a.scratch` null selects the
@@ -412,18 +355,16 @@ cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int warp_words_
                        long long slot_words_max = 0);
 
 #ifdef POLAR_SCL_KERNELS
-#define SCL_FOR_8(M, B) M(B + 0) M(B + 1) M(B + 2) M(B + 3) M(B + 4) M(B + 5) M(B + 6) M(B + 7)
-#define SCL_FOR_32(M) SCL_FOR_8(M, 0) SCL_FOR_8(M, 8) SCL_FOR_8(M, 16) SCL_FOR_8(M, 24)
-
 // One list step at an information bit: candidates, ranks, survivors.  Lane = path in and out;
 // returns the survivor's parent lane and decided bit, updates pm/act, reports duplication and
-// whether any survivor sits in another lane than its parent (`moved`, warp-uniform).
+// whether any survivor sits in another lane than its parent (`moved`, warp-uniform).  `ranked`: the
+// full-list shortcut is known to fail at this bit.
 template <bool TWO>
-__device__ __forceinline__ int scl_list_step(float lam, float& pm, int& act, int L, uint8_t* selc, uint32_t& bitv,
-                                             bool& dup, bool& moved)
+__device__ __forceinline__ int scl_list_step(float lam, float& pm, int& act, int L, uint8_t* selc, bool ranked,
+                                             uint32_t& bitv, bool& dup, bool& moved)
 {
     const int lane = threadIdx.x & 31;
-    if (act == L) {
+    if (act == L && !ranked) {
         // Full list: when every path's hard-decision child (metric pm) comes before every
         // penalised child (pm + |lambda|), the L survivors are exactly the hard-decision children,
         // in path order -- the same result as the ranking below, without it.  Metrics are >= +0,
@@ -526,20 +467,22 @@ __device__ __forceinline__ int scl_list_step(float lam, float& pm, int& act, int
 // survivors as scl_list_step, computed with loop bounds shared by both halves -- the fast path is
 // taken only when both lists qualify, and the ranks count over all 2L candidate slots with the
 // unused ones at +inf.  Returns the survivor's parent path (within the list).
-__device__ __forceinline__ int scl_list_step_half(float lam, float& pm, int& act, int L, uint8_t* selc,
+__device__ __forceinline__ int scl_list_step_half(float lam, float& pm, int& act, int L, uint8_t* selc, bool ranked,
                                                   uint32_t& bitv, bool& dup, bool& moved)
 {
     const Lanes<16> sg;
     const int pl = sg.pl;
-    const bool on = pl < act;
-    const uint32_t hd_max = sg.red_max(on ? __float_as_uint(pm) : 0u);
-    const uint32_t pen_min = sg.red_min(on ? __float_as_uint(__fadd_rn(pm, fabsf(lam))) : 0xffffffffu);
-    const bool fast = act == L && hd_max < pen_min;
-    if (__all_sync(0xffffffffu, fast || act == 0)) {
-        bitv = lam < 0.0f ? 1u : 0u;
-        dup = false;
-        moved = false;
-        return pl;
+    if (!ranked) {
+        const bool on = pl < act;
+        const uint32_t hd_max = sg.red_max(on ? __float_as_uint(pm) : 0u);
+        const uint32_t pen_min = sg.red_min(on ? __float_as_uint(__fadd_rn(pm, fabsf(lam))) : 0xffffffffu);
+        const bool fast = act == L && hd_max < pen_min;
+        if (__all_sync(0xffffffffu, fast || act == 0)) {
+            bitv = lam < 0.0f ? 1u : 0u;
+            dup = false;
+            moved = false;
+            return pl;
+        }
     }
     const int nc = 2 * act;
     const float inf = __int_as_float(0x7f800000);
@@ -588,11 +531,9 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
     const int lane = sg.pl;  // path of this lane within its list
     const int N = C.N, n = C.n, L = a.L;
     const float* y = a.llr + (frame < 0 ? 0 : (a.llr_off ? a.llr_off[frame] : (long long)frame * N));
+    const bool y16 = (reinterpret_cast<uintptr_t>(y) & 15u) == 0;
     uint32_t pA[2] = {0u, 0u}, pC[2] = {0u, 0u};  // upper-level pointer rows of path `lane`
     float pm = 0.0f;
-    // CRC syndrome of the path's decided bits so far: XOR of the syndrome columns of the positions
-    // decided 1 (frozen positions have column 0); survivors inherit their parent's
-    uint32_t syn = 0u;
     int act = frame < 0 ? 0 : 1;
     uint32_t shA = 0u, shC = 0u;  // upper levels that may be shared since the last duplication
     Leaf lf;
@@ -631,48 +572,68 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                 __syncthreads();
                 nact = nact_both = (int)ptab[96];
             }
-            const int cwk = scl_cs(k), total = nact << k, tmax = nact_both << k;
+            const int cwk = scl_cs(k);
             // element stride of a round: the list's lanes, or every thread of the CTA
             const int TW = MW ? (int)blockDim.x : W, tix = MW ? (int)threadIdx.x : lane;
-            // kSclUpRound elements per lane per round: all loads of a round are issued before any
-            // store, so the L2 latency of the upper levels (global for long lists) is paid once per
-            // round; the leaf registers are dead here and hold the round's values.  The loads are
-            // unconditional (an element past the list's end reads a valid slot: its path index is
-            // below L and its offset below len), so nothing but the stores is predicated and the
-            // rounds' independent chains interleave.
-            // CH: the level reads the channel row, whose values are staged as CA-SCL reads them
+            // Units of four consecutive elements of one path (a level has at least 32): one 16-byte
+            // load per operand and one set of pointers per unit.  kSclUpRound units per lane per
+            // round: all loads of a round are issued before any store, so the L2 latency of the
+            // upper levels (global for long lists) is paid once per round.  The loads are
+            // unconditional (a unit past the list's end reads a valid slot: its path index is below
+            // L and its offset below len), so nothing but the stores is predicated and the rounds'
+            // independent chains interleave.
+            // CH: the level reads the channel row, whose values are staged as CA-SCL reads them;
+            // the caller's row may start at any float, so its 16-byte loads need `y16`.
             auto rounds = [&](auto USE_G, auto FROM_CH) {
                 constexpr bool G = decltype(USE_G)::value, CH = decltype(FROM_CH)::value;
                 constexpr int U = kSclUpRound;
+                const int ku = k - 2, tot = nact << ku, tmax = nact_both << ku;
                 for (int e0 = 0; e0 < tmax; e0 += U * TW) {
-                    float va[U], vb[U];
+                    float4 va[U], vb[U];
                     uint32_t vw[U], pdv[U];
 #pragma unroll
                     for (int q = 0; q < U; ++q) {
                         const int e = e0 + TW * q + tix;
-                        const int p = (e >> k) & (W - 1);
+                        const int p = (e >> ku) & (W - 1);
                         pdv[q] = MW ? ptab[p] : sg.shfl(my_d, p);
-                        const uint32_t ps = MW ? ptab[32 + p] : sg.shfl(my_s, p);
-                        const int j = e & (len - 1);
-                        const float* src = srcb + ps * (2 * len);
-                        va[q] = src[j];
-                        vb[q] = src[j + len];
-                        if constexpr (CH) {
-                            va[q] = scl_stage(va[q]);
-                            vb[q] = scl_stage(vb[q]);
+                        const uint32_t ps = CH ? 0u : MW ? ptab[32 + p] : sg.shfl(my_s, p);
+                        const int j = (e << 2) & (len - 1);
+                        const float* src = srcb + ps * (2 * len) + j;
+                        if (CH && !y16) {
+                            va[q] = make_float4(src[0], src[1], src[2], src[3]);
+                            vb[q] = make_float4(src[len], src[len + 1], src[len + 2], src[len + 3]);
+                        } else {
+                            va[q] = *reinterpret_cast<const float4*>(src);
+                            vb[q] = *reinterpret_cast<const float4*>(src + len);
                         }
-                        if constexpr (G) vw[q] = cbk[(MW ? ptab[64 + p] : sg.shfl(my_c, p)) * cwk + (j >> 5)];
+                        if constexpr (G)
+                            vw[q] = cbk[(MW ? ptab[64 + p] : sg.shfl(my_c, p)) * cwk + (j >> 5)] >> (j & 31);
                     }
 #pragma unroll
                     for (int q = 0; q < U; ++q) {
                         const int e = e0 + TW * q + tix;
-                        const int j = e & (len - 1);
-                        float r;
+                        const int j = (e << 2) & (len - 1);
+                        float4 x = va[q], y4 = vb[q], r;
+                        if constexpr (CH) {
+                            x = make_float4(scl_stage(x.x), scl_stage(x.y), scl_stage(x.z), scl_stage(x.w));
+                            y4 = make_float4(scl_stage(y4.x), scl_stage(y4.y), scl_stage(y4.z), scl_stage(y4.w));
+                        }
                         if constexpr (G)
-                            r = scl_g(va[q], vb[q], (vw[q] >> (j & 31)) & 1u);
+                            r = make_float4(scl_g(x.x, y4.x, vw[q] & 1u), scl_g(x.y, y4.y, vw[q] & 2u),
+                                            scl_g(x.z, y4.z, vw[q] & 4u), scl_g(x.w, y4.w, vw[q] & 8u));
                         else
-                            r = xmin(va[q], vb[q]);
-                        if (e < total) dst[pdv[q] * dstride + j] = r;
+                            r = make_float4(xmin(x.x, y4.x), xmin(x.y, y4.y), xmin(x.z, y4.z), xmin(x.w, y4.w));
+                        if (e < tot) {
+                            float* d = dst + pdv[q] * dstride + j;
+                            if (stage) {  // staging rows have an odd stride
+                                d[0] = r.x;
+                                d[1] = r.y;
+                                d[2] = r.z;
+                                d[3] = r.w;
+                            } else {
+                                *reinterpret_cast<float4*>(d) = r;
+                            }
+                        }
                     }
                 }
             };
@@ -692,81 +653,152 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                 __syncwarp();
         }
         if (!lead) continue;  // the helper warps only share the upper levels
-        // level 5 of every path into its lane's registers (lanes past the list read row 0: the
-        // staging area has L rows); the lower leaf levels and partial sums start afresh (every bit
-        // of the block writes them before reading them), which also tells the compiler that their
-        // registers were free during the upper-level rounds above
-        {
-            const float* row = S.stage + (lane < L ? lane : 0) * kSclStage;
-#pragma unroll
-            for (int j = 0; j < 32; ++j) lf.l5[j] = row[j];
-#pragma unroll
-            for (int j = 0; j < 16; ++j) lf.l4[j] = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 8; ++j) lf.l3[j] = 0.0f;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) lf.l2[j] = 0.0f;
-            lf.l1[0] = lf.l1[1] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < 5; ++k) lf.c[k] = 0u;
-        }
         // ------------------------------------------------ the 32 bits of the block
-        // A runtime loop: one copy of the list step serves all 32 bits, and only the per-bit leaf
-        // code (whose register indices are compile-time constants) is dispatched by the bit index.
-        // Unrolling the block with a list step inlined per bit overflowed the instruction cache.
+        // A runtime walk of the block's tree, four bits at a time; one copy of the list step serves
+        // all bits (unrolling it per bit overflowed the instruction cache).  Lanes past the list
+        // read row 0 (the staging area has L rows) and compute values nobody reads.
         const uint32_t fw = C.frozen_bits[blk], dw = C.decided_bits[blk];
         uint32_t v5 = 0u;
+        lf.row = lane < L ? lane : 0;
+        int r = 0, failed = -1;  // failed: bit at which the full-list shortcut is known to fail
+        if (fw == 0u) {
+            const float* row = S.stage + lf.row * kSclStage;
+            if (leaf_all_hard<W, 32>(sg, [&](int j) { return row[j]; }, pm, act, L, v5)) r = 32;
+            else failed = 0;
+        }
 #pragma unroll 1
-        for (int r = 0; r < 32; ++r) {
-            const uint32_t col = C.colsyn[blk * 32 + r];
-            float lam = 0.0f;
-            if (r & 1) {
-                // odd bits (half of them): one g from level 1, no dispatch
-                lam = scl_g(lf.l1[0], lf.l1[1], lf.c[0] & 1u);
-            } else if ((r & 3) == 2) {
-                // bits 2 mod 4 (a quarter): g into level 1, then f
-                leaf_g<2>(lf.l2, lf.l1, lf.c[1]);
-                lam = xmin(lf.l1[0], lf.l1[1]);
-            } else if ((r & 7) == 4) {
-                // bits 4 mod 8 (an eighth): g into level 2, then f twice
-                leaf_g<4>(lf.l3, lf.l2, lf.c[2]);
-                leaf_f<2>(lf.l2, lf.l1);
-                lam = xmin(lf.l1[0], lf.l1[1]);
-            } else {
-                switch (r) {
-#define SCL_LEAF_LLR(R) \
-    case 8 * (R): lam = leaf_llr<8 * (R)>(lf); break;
-                    SCL_LEAF_LLR(0) SCL_LEAF_LLR(1) SCL_LEAF_LLR(2) SCL_LEAF_LLR(3)
-#undef SCL_LEAF_LLR
+        while (r < 32) {
+            uint32_t v = 0u;
+            int k = 5;  // level of the node decided by this step; 5: none yet
+            if ((r & 15) == 0) {
+                const float* row = S.stage + lf.row * kSclStage;
+                if (r == 0) {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) lf.l4[j] = xmin(row[j], row[j + 16]);
+                } else {
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) lf.l4[j] = scl_g(row[j], row[j + 16], lf.c[4] & (1u << j));
+                }
+                const uint32_t f = (fw >> r) & 0xffffu;
+                if (f == 0xffffu) {
+                    leaf_frozen(lf.l4, pm);
+                    k = 4;
+                } else if (f == 0u && failed != r) {
+                    if (leaf_all_hard<W, 16>(sg, [&](int j) { return lf.l4[j]; }, pm, act, L, v)) k = 4;
+                    else failed = r;
                 }
             }
-            uint32_t bitv = 0u;
-            bool moved = false;
-            int parent = lane;
-            if ((fw >> r) & 1u) {
-                if (lane < act && lam < 0.0f) pm = __fadd_rn(pm, fabsf(lam));
-            } else if ((dw >> r) & 1u) {
-                // decision aiding: each path takes its hard decision, no branching, no metric
-                bitv = lam < 0.0f ? 1u : 0u;
-            } else {
-                bool dup = false;
-                if constexpr (W == 32)
-                    parent = scl_list_step<TWO>(lam, pm, act, L, selc, bitv, dup, moved);
+            if (k == 5 && (r & 7) == 0) {
+                if (r & 8)
+                    leaf_g<8>(lf.l4, lf.l3, lf.c[3]);
                 else
-                    parent = scl_list_step_half(lam, pm, act, L, selc, bitv, dup, moved);
-                if (moved) {
-                    const int src = sg.base + parent;
-                    leaf_inherit_rt(lf, src, leaf_live_mask(r));
-                    pA[0] = __shfl_sync(0xffffffffu, pA[0], src);
-                    pA[1] = __shfl_sync(0xffffffffu, pA[1], src);
-                    pC[0] = __shfl_sync(0xffffffffu, pC[0], src);
-                    pC[1] = __shfl_sync(0xffffffffu, pC[1], src);
-                    syn = __shfl_sync(0xffffffffu, syn, src);
+                    leaf_f<8>(lf.l4, lf.l3);
+                const uint32_t f = (fw >> r) & 0xffu;
+                if (f == 0xffu) {
+                    leaf_frozen(lf.l3, pm);
+                    k = 3;
+                } else if (f == 0u && failed != r) {
+                    if (leaf_all_hard<W, 8>(sg, [&](int j) { return lf.l3[j]; }, pm, act, L, v)) k = 3;
+                    else failed = r;
                 }
-                if (dup) shA = shC = 0xffffffffu;
             }
-            if (bitv) syn ^= col;
-            v5 = leaf_psum_rt(lf, bitv, r);
+            if (k == 5) {
+                if (r & 4)
+                    leaf_g<4>(lf.l3, lf.l2, lf.c[2]);
+                else
+                    leaf_f<4>(lf.l3, lf.l2);
+                const uint32_t f = (fw >> r) & 0xfu;
+                k = 2;
+                bool whole = false;
+                if (f == 0xfu) {
+                    leaf_frozen(lf.l2, pm);
+                    whole = true;
+                } else if (f == 0u && failed != r) {
+                    whole = leaf_all_hard<W, 4>(sg, [&](int j) { return lf.l2[j]; }, pm, act, L, v);
+                    if (!whole) failed = r;
+                }
+                if (!whole) {
+                    // bit by bit
+#pragma unroll 1
+                    for (int q = r; q < r + 4; ++q) {
+                        float lam;
+                        if (q & 1) {
+                            lam = scl_g(lf.l1[0], lf.l1[1], lf.c[0] & 1u);
+                        } else {
+                            if (q & 2)
+                                leaf_g<2>(lf.l2, lf.l1, lf.c[1]);
+                            else
+                                leaf_f<2>(lf.l2, lf.l1);
+                            lam = xmin(lf.l1[0], lf.l1[1]);
+                        }
+                        uint32_t bitv = 0u;
+                        if ((fw >> q) & 1u) {
+                            pm = __fsub_rn(pm, fminf(lam, 0.0f));
+                        } else if ((dw >> q) & 1u) {
+                            // decision aiding: each path takes its hard decision, no branching, no metric
+                            bitv = lam < 0.0f ? 1u : 0u;
+                        } else {
+                            bool dup = false, moved = false;
+                            int parent;
+                            if constexpr (W == 32)
+                                parent = scl_list_step<TWO>(lam, pm, act, L, selc, failed == q, bitv, dup, moved);
+                            else
+                                parent = scl_list_step_half(lam, pm, act, L, selc, failed == q, bitv, dup, moved);
+                            if (moved) {
+                                const int src = sg.base + parent;
+                                if (!(q & 8)) leaf_copy<16>(lf.l4, src);
+                                if (!(q & 4)) leaf_copy<8>(lf.l3, src);
+                                if (!(q & 2)) leaf_copy<4>(lf.l2, src);
+                                if (!(q & 1)) leaf_copy<2>(lf.l1, src);
+#pragma unroll
+                                for (int i = 0; i < 5; ++i)
+                                    if (q & (1 << i)) lf.c[i] = __shfl_sync(0xffffffffu, lf.c[i], src);
+                                lf.row = __shfl_sync(0xffffffffu, lf.row, src);
+                                pA[0] = __shfl_sync(0xffffffffu, pA[0], src);
+                                pA[1] = __shfl_sync(0xffffffffu, pA[1], src);
+                                pC[0] = __shfl_sync(0xffffffffu, pC[0], src);
+                                pC[1] = __shfl_sync(0xffffffffu, pC[1], src);
+                            }
+                            if (dup) shA = shC = 0xffffffffu;
+                        }
+                        // partial sums of levels 0..1; the last bit completes the node's codeword
+                        if (!(q & 1)) {
+                            lf.c[0] = bitv;
+                        } else {
+                            const uint32_t v1 = (bitv ^ lf.c[0]) | (bitv << 1);
+                            if (q & 2)
+                                v = (v1 ^ lf.c[1]) | (v1 << 2);
+                            else
+                                lf.c[1] = v1;
+                        }
+                    }
+                }
+            }
+            // the node of 2^k bits at r has codeword v: fold it into its ancestors
+            const int r0 = r;
+            r += 1 << k;
+            if (k == 2) {
+                if (r0 & 4) {
+                    v = (v ^ lf.c[2]) | (v << 4);
+                    k = 3;
+                } else {
+                    lf.c[2] = v;
+                }
+            }
+            if (k == 3) {
+                if (r0 & 8) {
+                    v = (v ^ lf.c[3]) | (v << 8);
+                    k = 4;
+                } else {
+                    lf.c[3] = v;
+                }
+            }
+            if (k == 4) {
+                if (r0 & 16)
+                    v5 = (v ^ lf.c[4]) | (v << 16);
+                else
+                    lf.c[4] = v;
+            }
         }
         // ------------------------------------------------ block complete: partial sums upward
         {
@@ -835,37 +867,37 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
     }
     if (!lead) return;
     // ------------------------------------------------------------------ CRC selection
-    // Each path's syndrome was accumulated bit by bit; the chosen path's codeword (level-n array)
-    // is turned into u = x G in place for the output.  The list's lanes hold the codeword's 32-bit
-    // words lane + W h.
+    // The paths in (metric, index) order: the codeword x of each (its level-n array; the list's
+    // lanes hold the 32-bit words lane + W h) is turned into u = x G and its CRC syndrome, the XOR
+    // of the syndrome columns of the positions decided 1, is formed with one column per lane.  The
+    // first path whose syndrome is zero is output, the best one if none is.  On most frames that is
+    // one path's work, against a column load and XOR per path and bit, and a shuffle per list step,
+    // for syndromes kept along the way.
     constexpr int H = kMaxWords / W;  // words per lane
     const int words = N >> 5;
     uint32_t* xl = S.Cl(n);
     const uint32_t my_x = fld(pC, n);
-    const uint32_t synd = lane < act ? syn : 0xffffffffu;  // lane p: syndrome of path p
+    const uint32_t m[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
+    uint32_t best[H];   // u of the output path,
+    uint32_t* uw = xl;  // written back over its codeword, where the payload bits are picked from
+    bool avail = lane < act, done = act == 0, any_ok = false, first = true;
     __syncwarp();
-    // first CRC-passing path in (metric, index) order, else the best metric
-    const bool ok_lane = lane < act && synd == 0u;
-    const bool any_ok = sg.ballot(ok_lane) != 0u;
-    const bool cand = any_ok ? ok_lane : lane < act;
-    float key = cand ? pm : __int_as_float(0x7f800000);
-    int who = cand ? lane : 64;
+    while (__any_sync(0xffffffffu, !done)) {
+        float key = avail ? pm : __int_as_float(0x7f800000);
+        int who = avail ? lane : 64;
 #pragma unroll
-    for (int off = W / 2; off >= 1; off >>= 1) {
-        const float ok2 = __shfl_xor_sync(0xffffffffu, key, off);
-        const int ow = __shfl_xor_sync(0xffffffffu, who, off);
-        if (ok2 < key || (ok2 == key && ow < who)) {
-            key = ok2;
-            who = ow;
+        for (int off = W / 2; off >= 1; off >>= 1) {
+            const float ok2 = __shfl_xor_sync(0xffffffffu, key, off);
+            const int ow = __shfl_xor_sync(0xffffffffu, who, off);
+            if (ok2 < key || (ok2 == key && ow < who)) {
+                key = ok2;
+                who = ow;
+            }
         }
-    }
-    uint32_t* uw = xl + sg.shfl(my_x, who & (W - 1)) * scl_cs(n);
-    {
-        const bool live = frame >= 0;
+        uint32_t* xw = xl + sg.shfl(my_x, who & (W - 1)) * scl_cs(n);
         uint32_t w[H];
 #pragma unroll
-        for (int h = 0; h < H; ++h) w[h] = (live && lane + W * h < words) ? uw[lane + W * h] : 0u;
-        const uint32_t m[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
+        for (int h = 0; h < H; ++h) w[h] = (frame >= 0 && lane + W * h < words) ? xw[lane + W * h] : 0u;
 #pragma unroll
         for (int h = 0; h < H; ++h)
 #pragma unroll
@@ -883,11 +915,39 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
             for (int h = 0; h < H; ++h)
                 if (!(h & hd) && (h | hd) < H) w[h] ^= w[h | hd];
         }
+        uint32_t syn = 0u;
+#pragma unroll
+        for (int h = 0; h < H; ++h) {
+            const int cnt = min(W, words - W * h);
+            const uint32_t* col = C.colsyn + W * h * 32 + lane;
+#pragma unroll 4
+            for (int i = 0; i < cnt; ++i) {
+                const uint32_t ui = sg.shfl(w[h], i);
+#pragma unroll
+                for (int z = 0; z < 32; z += W)
+                    if ((ui >> (lane + z)) & 1u) syn ^= col[32 * i + z];
+            }
+        }
+        syn = sg.red_xor(syn);
+        if (!done) {
+            any_ok = syn == 0u;
+            if (first || any_ok) {
+#pragma unroll
+                for (int h = 0; h < H; ++h) best[h] = w[h];
+                uw = xw;
+            }
+            first = false;
+            if (lane == who) avail = false;
+        }
+        const bool none_left = sg.ballot(avail) == 0u;
+        done = done || any_ok || none_left;
+    }
+    if (frame >= 0) {
 #pragma unroll
         for (int h = 0; h < H; ++h)
-            if (live && lane + W * h < words) uw[lane + W * h] = w[h];
-        __syncwarp();
+            if (lane + W * h < words) uw[lane + W * h] = best[h];
     }
+    __syncwarp();
     if (frame >= 0) {
         uint8_t* out = a.bits + (size_t)frame * a.row_bytes;
         for (int by = lane; by < a.row_bytes; by += W) {
@@ -926,9 +986,10 @@ __device__ __forceinline__ void scl_warp_frame(const SCLArgs& a, int frame, int 
         S.KS = a.KS;
         S.KC = a.KC;
     }
-    S.sC = ws;
-    S.sA = reinterpret_cast<float*>(ws + scl_smem_c_words(S.KC, L));
+    // the LLR levels first: their 16-byte accesses need the list's 16-byte aligned start
+    S.sA = reinterpret_cast<float*>(ws);
     S.stage = S.sA + scl_smem_llr_words(S.KS, L);
+    S.sC = reinterpret_cast<uint32_t*>(S.stage + L * kSclStage);
     S.gA = slot;
     S.gC = slot ? reinterpret_cast<uint32_t*>(slot + (size_t)L * (C.N - (2 << S.KS))) : nullptr;
     scl_decode_frame<TWO, W, MW>(a, C, frame, S, selc, ptab);
@@ -938,7 +999,7 @@ __device__ __forceinline__ void scl_warp_frame(const SCLArgs& a, int frame, int 
 // batch (frames sorted by code) the two frames of a pair normally share their code; a pair whose
 // codes differ is decoded one list after the other.
 template <bool TWO, int W>
-__global__ void __launch_bounds__(kSclWarpsPerCTA * 32) scl_kernel(const SCLArgs a)
+__global__ void __launch_bounds__(kSclWarpsPerCTA * 32, 4) scl_kernel(const SCLArgs a)
 {
     constexpr int LISTS = 32 / W;
     extern __shared__ __align__(16) uint32_t smem[];
@@ -979,22 +1040,20 @@ __global__ void __launch_bounds__(kSclWarpsPerCTA * 32) scl_kernel(const SCLArgs
         if (idx >= count) break;  // uniform over the warp
         const int k = idx + li;
         const int frame = k < count ? (a.list ? a.list[k] : k) : -1;
-        if (!a.code_of) {
-            scl_warp_frame<TWO, W>(a, frame, -1, ws, slot, selc);
-            continue;
-        }
-        const int cf = frame >= 0 ? a.code_of[frame] : -1;
+        // one call site: every inlined copy of the decoder would be scheduled and allocated apart
+        int code = a.code_of && frame >= 0 ? a.code_of[frame] : -1, passes = 1;
+        int other = -1;
         if constexpr (LISTS == 2) {
-            const int c0 = __shfl_sync(0xffffffffu, cf, 0), c1 = __shfl_sync(0xffffffffu, cf, 16);
-            if (c0 >= 0 && c1 >= 0 && c0 != c1) {
-                scl_warp_frame<TWO, W>(a, li == 0 ? frame : -1, c0, ws, slot, selc);
-                scl_warp_frame<TWO, W>(a, li == 1 ? frame : -1, c1, ws, slot, selc);
-            } else {
-                scl_warp_frame<TWO, W>(a, frame, c0 >= 0 ? c0 : c1, ws, slot, selc);
+            if (a.code_of) {
+                const int c0 = __shfl_sync(0xffffffffu, code, 0), c1 = __shfl_sync(0xffffffffu, code, 16);
+                passes = c0 >= 0 && c1 >= 0 && c0 != c1 ? 2 : 1;
+                code = c0 >= 0 ? c0 : c1;
+                other = c1;
             }
-        } else {
-            scl_warp_frame<TWO, W>(a, frame, cf, ws, slot, selc);
         }
+#pragma unroll 1
+        for (int q = 0; q < passes; ++q)
+            scl_warp_frame<TWO, W>(a, passes == 1 || li == q ? frame : -1, q ? other : code, ws, slot, selc);
     }
 }
 
@@ -1009,7 +1068,16 @@ cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int warp_words_
     a.KC = p.KC;
     a.list_words = std::max(p.list_words, warp_words_max - 16);
     a.warp_words = lists * a.list_words + 16;
-    a.slot_words = std::max(p.slot_words, slot_words_max);
+    // slots hold 16-byte vectors: each starts on a 16-byte boundary, wherever the caller's workspace
+    // starts, so the same scratch bytes may give a few slots less than it was sized for
+    const long long slot_words = std::max(p.slot_words, slot_words_max);
+    a.slot_words = (slot_words + 3) / 4 * 4;
+    long long slots = (long long)scl_sm_count() * kSclWarpsPerSM;
+    if (!all_smem && slot_words > 0) {
+        const long long skip = (long long)((16 - (reinterpret_cast<uintptr_t>(a.scratch) & 15)) & 15) / 4;
+        a.scratch += skip;
+        slots = (slots * slot_words - skip) / a.slot_words;
+    }
     int W = kSclWarpsPerCTA;
     const size_t wb = (size_t)a.warp_words * 4;
     while (W > 1 && (size_t)W * wb > 200 * 1024) W >>= 1;
@@ -1025,7 +1093,7 @@ cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int warp_words_
     if (per_sm < 1) return cudaErrorInvalidConfiguration;
     const int sms = scl_sm_count();
     long long grid = (long long)sms * per_sm;
-    if (!all_smem) grid = std::min<long long>(grid, (long long)sms * kSclWarpsPerSM / (W * lists));
+    if (!all_smem) grid = std::min<long long>(grid, slots / (W * lists));
     if (!a.list) {
         // known work: whole-warp lists with at most one frame per CTA of the full grid get a CTA
         // per frame (its warps then share each frame's upper levels), otherwise no idle CTAs
