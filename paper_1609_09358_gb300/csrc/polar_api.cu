@@ -921,9 +921,11 @@ static int wms_common(const polar_code* code, const float* llr, int B, int T, fl
     a.T = T;
     a.M = llr_max;
     a.w = w;
-    a.store = static_cast<float*>(workspace);
-    a.adj = a.store + (size_t)B * 2 * T * n * N;
+    // the stored columns take 2 (n-1) N floats per frame and iteration, 16-byte aligned; the rest of
+    // the workspace is unused
+    a.store = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(workspace), 16));
     a.code = d;
+    a.w16 = (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
     return POLAR_OK;
 }
 
@@ -938,8 +940,8 @@ int wms_forward(const polar_code* code, const float* llr, int32_t B, int32_t T, 
     if (!llr_u) return fail(POLAR_ERR_ARG, "NULL llr_u");
     a.all = all_iters ? 1 : 0;
     a.llr_u = llr_u;
-    wms_forward_kernel<<<B, code->N / 2, 0, st>>>(a);
-    POLAR_CUDA(cudaGetLastError());
+    a.out16 = (reinterpret_cast<uintptr_t>(llr_u) & 15u) == 0;
+    POLAR_CUDA(wms_forward_launch(log2i(code->N), a, st));
     return POLAR_OK;
 }
 
@@ -959,8 +961,9 @@ int wms_backward(const polar_code* code, const float* llr, int32_t B, int32_t T,
     a.all = all_iters ? 1 : 0;
     a.grad_u = grad_llr_u;
     a.grad_w = grad_w;
-    wms_backward_kernel<<<B, code->N / 2, 0, st>>>(a);
-    POLAR_CUDA(cudaGetLastError());
+    a.out16 = (reinterpret_cast<uintptr_t>(grad_llr_u) & 15u) == 0;
+    a.gw16 = (reinterpret_cast<uintptr_t>(grad_w) & 15u) == 0;
+    POLAR_CUDA(wms_backward_launch(log2i(code->N), a, st));
     return POLAR_OK;
 }
 
