@@ -559,10 +559,17 @@ int polar_encode(const polar_code* code, const uint8_t* payload, int32_t B, uint
     if (rc) return rc;
     if (B == 0) return POLAR_OK;
     if (!codeword || (!payload && code->K > code->crc_len)) return fail(POLAR_ERR_ARG, "NULL payload/codeword");
-    const int warps = 4;
-    encode_kernel<<<(B + warps - 1) / warps, warps * 32, 0, st>>>(d, payload, B, (code->K - code->crc_len + 7) / 8,
-                                                                codeword);
-    POLAR_CUDA(cudaGetLastError());
+    // enough CTAs for several per SM; each loops over the batch and prepares the code's tables once
+    const int N = code->N, P = code->K - code->crc_len, per_cta = kEncWarps * (N >= 1024 ? 1 : 1024 / N);
+    const int grid = std::min((B + per_cta - 1) / per_cta, 4 * scl_sm_count());
+    const size_t smem = enc_smem_bytes(N, P);
+    const void* fn = N <= 1024   ? (const void*)encode_kernel<1>
+                     : N == 2048 ? (const void*)encode_kernel<2>
+                                 : (const void*)encode_kernel<4>;
+    if (smem > 48 * 1024) POLAR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int pay_bytes = (P + 7) / 8;
+    void* args[] = {&d, &payload, &B, &pay_bytes, &codeword};
+    POLAR_CUDA(cudaLaunchKernel(fn, dim3(grid), dim3(kEncWarps * 32), args, smem, st));
     return POLAR_OK;
 }
 
@@ -571,9 +578,12 @@ int polar_random_payload(int32_t B, int32_t P, uint64_t seed, uint64_t frame0, u
     if (B < 0 || P < 0) return fail(POLAR_ERR_ARG, "B or P < 0");
     if (B == 0 || P == 0) return POLAR_OK;
     if (!payload) return fail(POLAR_ERR_ARG, "NULL payload");
-    const long long total = (long long)B * (((P + 31) / 32 + 3) / 4);
-    random_payload_kernel<<<(unsigned)((total + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        B, P, seed, frame0, payload);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    const long long bytes = ((long long)P + 7) / 8, total = B * (((long long)P + 127) / 128);
+    if (bytes <= kPayMaxBytes)
+        random_payload_kernel<<<(B + kPayRows - 1) / kPayRows, 256, kPayRows * bytes, st>>>(B, P, seed, frame0, payload);
+    else
+        random_payload_direct_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, P, seed, frame0, payload);
     POLAR_CUDA(cudaGetLastError());
     return POLAR_OK;
 }
@@ -587,7 +597,7 @@ int polar_awgn_llr(const uint8_t* codeword, int32_t B, int32_t N, float sigma, c
     if (!codeword || !llr) return fail(POLAR_ERR_ARG, "NULL codeword/llr");
     const long long total = (long long)B * (N / 4);
     awgn_llr_kernel<<<(unsigned)((total + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        codeword, B, N, sigma, sigma_per_frame, seed, frame0, llr);
+        codeword, B, log2i(N), sigma, sigma_per_frame ? 0.0f : 2.0f / (sigma * sigma), sigma_per_frame, seed, frame0, llr);
     POLAR_CUDA(cudaGetLastError());
     return POLAR_OK;
 }
@@ -914,7 +924,6 @@ static int wms_common(const polar_code* code, const float* llr, int B, int T, fl
     if (B > 0 && (!workspace || ws < need)) return fail(POLAR_ERR_WORKSPACE, "workspace %zu < %zu bytes", ws, need);
     const DevCode* d = nullptr;
     if ((rc = code_slot(code, st, &d))) return rc;
-    const size_t n = (size_t)log2i(code->N), N = (size_t)code->N;
     a = WMSArgs{};
     a.llr = llr;
     a.B = B;
