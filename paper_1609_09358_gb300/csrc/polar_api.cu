@@ -1004,7 +1004,7 @@ MixLayout mix_layout(int ncodes, int B, size_t scratch_bytes)
     return m;
 }
 
-int mix_check(const polar_code* codes, int ncodes, int B, int L, int row_stride, int* max_row, int* warp_words,
+int mix_check(const polar_code* codes, int ncodes, int B, int L, int row_stride, int* max_row, int* list_words,
               long long* slot_words)
 {
     if (!codes || ncodes < 1 || ncodes > POLAR_MAX_MIX_CODES)
@@ -1019,16 +1019,16 @@ int mix_check(const polar_code* codes, int ncodes, int B, int L, int row_stride,
             return fail(POLAR_ERR_ARG, "mixed batches: N = %d > %d", codes[c].N, POLAR_MAX_N_MIXED);
         mr = std::max(mr, (codes[c].K - codes[c].crc_len + 7) / 8);
         if (L > 0) {
-            // per-list words (+ the warp's 16 scratch words) and global slot of the CA-SCL launch's
+            // per-list shared words and global slot of the CA-SCL launch's
             // list width (two lists per warp for L <= 8)
             const SCLPlan p = scl_plan(codes[c].N, L, false, scl_two_lists(L, false) ? 2 : 1);
-            ww = std::max(ww, p.list_words + 16);
+            ww = std::max(ww, p.list_words);
             sw = std::max(sw, p.slot_words);
         }
     }
     if (row_stride >= 0 && row_stride < mr) return fail(POLAR_ERR_ARG, "row_stride %d < %d bytes", row_stride, mr);
     if (max_row) *max_row = mr;
-    if (warp_words) *warp_words = ww;
+    if (list_words) *list_words = ww;
     if (slot_words) *slot_words = sw;
     return POLAR_OK;
 }

@@ -84,12 +84,14 @@ struct SCLPlan {
     int warp_words, list_words;
     long long slot_words;
 };
-// Level 5 of every path is computed element-parallel into a staging row per path (33 words: the
-// pad makes both the warp's row-wise writes and the lanes' per-path reads bank-conflict free) and
-// then read into the path's registers.
-constexpr int kSclStage = 33;
-// units (of four elements) per lane and round of the element-parallel upper-level updates
-constexpr int kSclUpRound = 2;
+// Level 5 of a path is computed by its lane from the path's level-6 array, which is always in shared
+// memory, and kept in a staging row of 32 words.  Both are read and written by 32 lanes at a time, each
+// in its own row, 16 bytes per access: the 16-byte chunk index is XORed with the row number modulo 8,
+// which spreads eight rows over all banks.
+constexpr int kSclStage = 32;
+__host__ __device__ inline int scl_chunk(int row, int chunk) { return (chunk ^ (row & 7)) << 2; }  // word offset
+// per warp: 16 words of list-step scratch, then the packed path pointers of a level and the path count
+constexpr int kSclScratch = 16, kSclPtrs = 40, kSclWarpWords = kSclScratch + kSclPtrs;
 __host__ __device__ inline long long scl_smem_llr_words(int KS, int L) { return KS >= 6 ? (long long)L * ((2 << KS) - 64) : 0; }
 __host__ __device__ inline long long scl_smem_c_words(int KC, int L) { return KC >= 5 ? (long long)L * (scl_cssum(KC + 1) - 5) : 0; }
 // `lists` = frames per warp (1, or 2 with half-warp lists): the shared-memory budget of a frame
@@ -102,18 +104,17 @@ __host__ __device__ inline SCLPlan scl_plan(int N, int L, bool all_smem, int lis
         p.KS = n - 1;
         p.KC = n;
     } else {
-        p.KS = 5;
-        // up to 6 KB of LLR levels per frame (8 KB, which puts level 6 of a 32-path list in shared
-        // memory, measured 3% slower for a single frame and 3% faster for 2^16 frames: not kept)
+        p.KS = 6;
+        // up to 6 KB of LLR levels per frame, at least level 6
         while (p.KS + 1 <= n - 1 && 4 * scl_smem_llr_words(p.KS + 1, L) * lists <= 6144) ++p.KS;
         p.KC = 4;
         while (p.KC + 1 <= n && 4 * scl_smem_c_words(p.KC + 1, L) * lists <= 2048) ++p.KC;
     }
-    // per list: [LLR levels 6..KS][level-5 staging, L rows of 33 words][C levels 5..KC]; per warp:
-    // the lists, then 16 words of list-step scratch
+    // per list: [LLR levels 6..KS][level-5 staging, L rows of 32 words][C levels 5..KC]; per warp:
+    // the lists, then kSclWarpWords words of scratch
     p.list_words = (int)(scl_smem_llr_words(p.KS, L) + scl_smem_c_words(p.KC, L)) + L * kSclStage;
     p.list_words = (p.list_words + 3) & ~3;
-    p.warp_words = lists * p.list_words + 16;
+    p.warp_words = lists * p.list_words + kSclWarpWords;
     p.slot_words = (long long)L * (N - (2 << p.KS)) + (long long)L * (scl_cssum(n + 1) - scl_cssum(p.KC + 1));
     return p;
 }
@@ -239,12 +240,17 @@ __device__ __forceinline__ void scl_own(uint32_t (&w)[2], int k, int act, int L)
     uint32_t freem = ~used & (L >= 32 ? 0xffffffffu : ((1u << L) - 1u));
     const int r = __popc(sg.ballot(need) & below);
     if (need) {
+#pragma unroll 1
         for (int q = 0; q < r; ++q) freem &= freem - 1u;  // drop the r lowest free arrays
         set_fld(w, k, (uint32_t)(__ffs(freem) - 1));
     }
 }
 
-__device__ __forceinline__ float scl_g(float a, float b, uint32_t v) { return v ? __fsub_rn(b, a) : __fadd_rn(b, a); }
+// g = b + (1 - 2v) a with v = bit j of c: a's sign flipped by the bit (b - a and b + (-a) are the same)
+__device__ __forceinline__ float scl_g(float a, float b, uint32_t c, int j)
+{
+    return __fadd_rn(b, __uint_as_float(__float_as_uint(a) ^ ((c << (31 - j)) & 0x80000000u)));
+}
 
 struct SCLWarp {
     float* stage;  // shared level-5 staging rows [L][kSclStage]
@@ -276,7 +282,7 @@ template <int LEN>
 __device__ __forceinline__ void leaf_g(const float (&src)[2 * LEN], float (&dst)[LEN], uint32_t c)
 {
 #pragma unroll
-    for (int j = 0; j < LEN; ++j) dst[j] = scl_g(src[j], src[j + LEN], (c >> j) & 1u);
+    for (int j = 0; j < LEN; ++j) dst[j] = scl_g(src[j], src[j + LEN], c, j);
 }
 template <int LEN>
 __device__ __forceinline__ void leaf_copy(float (&a)[LEN], int parent)
@@ -319,8 +325,9 @@ __device__ __forceinline__ void leaf_frozen(const float (&a)[LEN], float& pm)
 // are the paths themselves with the sign bits of a as the node's codeword.  If the condition
 // fails, the first bit's shortcut fails as well.  (A zero LLR makes m = 0 and fails it, so the
 // signs are those of nonzero values.)
-template <int W, int LEN, class Get>
-__device__ __forceinline__ bool leaf_all_hard(const Lanes<W>& sg, Get a, float pm, int act, int L, uint32_t& v)
+template <int W, int LEN>
+__device__ __forceinline__ bool leaf_all_hard(const Lanes<W>& sg, const float (&a)[LEN], float pm, int act, int L,
+                                              uint32_t& v)
 {
     if constexpr (W == 32) {
         if (act != L) return false;
@@ -331,7 +338,7 @@ __device__ __forceinline__ bool leaf_all_hard(const Lanes<W>& sg, Get a, float p
     v = 0u;
 #pragma unroll
     for (int j = LEN - 1; j >= 0; --j) {
-        const float x = a(j);
+        const float x = a[j];
         v = __funnelshift_l(__float_as_uint(x), v, 1);
         constexpr int Q = LEN >= 4 ? 4 : LEN;
         m[j % Q] = j + Q >= LEN ? fabsf(x) : fminf(m[j % Q], fabsf(x));
@@ -349,9 +356,9 @@ __device__ __forceinline__ bool leaf_all_hard(const Lanes<W>& sg, Get a, float p
 }
 
 // Launches the persistent CA-SCL grid (defined in scl_launch.cu).  `a.scratch` null selects the
-// all-shared-memory layout; warp_words_max / slot_words_max widen the per-warp storage for mixed
+// all-shared-memory layout; list_words_max / slot_words_max widen the per-warp storage for mixed
 // batches.
-cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int warp_words_max = 0,
+cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int list_words_max = 0,
                        long long slot_words_max = 0);
 
 #ifdef POLAR_SCL_KERNELS
@@ -517,16 +524,23 @@ __device__ __forceinline__ int scl_list_step_half(float lam, float& pm, int& act
 
 // Decode one frame per list: the warp's frame (W = 32), or each half-warp's frame (W = 16; a
 // half without a frame passes frame < 0 and decodes nothing).  TWO: L = 32, two candidates per
-// lane.  MW: every warp of the CTA calls with the same frame; warp 0 holds the list and runs the
-// bit loop, and all warps share the element-parallel upper-level updates (their path pointers
-// and path count passed through `ptab`, 104 shared words), with CTA barriers around each level.
-template <bool TWO, int W, bool MW = false>
+// lane.  mw (W = 32): every warp of the CTA calls with the same frame; warp 0 holds the list and runs
+// the bit loop, and all warps share the element-parallel upper-level updates, with CTA barriers
+// around each level.  W = 32 passes the path pointers of a level through `ptab` (kSclPtrs words; mw:
+// warp 0's), W = 16 by shuffles.  (mw is a run-time flag and everything done once per frame is a loop:
+// the body is long, and with 16 warps at different places of it instruction fetch is a top stall.)
+template <bool TWO, int W>
 __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, const SCLWarp& S, uint8_t* selc,
-                                 uint32_t* ptab = nullptr)
+                                 uint32_t* ptab, const bool mw)
 {
     static_assert(W == 32 || !TWO, "half-warp lists hold at most 8 paths");
-    static_assert(!MW || W == 32, "the multi-warp form takes whole-warp lists");
-    const bool lead = !MW || threadIdx.x < 32;
+    const bool lead = !mw || threadIdx.x < 32;
+    auto level_sync = [&]() {
+        if (W == 32 && mw)
+            __syncthreads();
+        else
+            __syncwarp();
+    };
     const Lanes<W> sg;
     const int lane = sg.pl;  // path of this lane within its list
     const int N = C.N, n = C.n, L = a.L;
@@ -543,63 +557,68 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
     for (int blk = 0; blk < nblocks; ++blk) {
         // ------------------------------------------------ upper levels on entering the block
         const int t = blk == 0 ? n : 5 + __ffs(blk) - 1;
-        const int top = blk == 0 ? n - 1 : t;
         const int act_both = sg.both_max(act);
-        for (int k = top; k >= 5; --k) {
-            // level 5 goes to the staging rows (indexed by path), levels >= 6 to their arrays
-            const bool stage = k == 5;
-            if (lead && !stage && __any_sync(0xffffffffu, (shA >> k) & 1u)) {
-                scl_own<W>(pA, k, act, L);
-                shA &= ~(1u << k);
+        // element stride of a round: the list's lanes, or every thread of the CTA
+        const int TW = W == 32 && mw ? (int)blockDim.x : W, tix = W == 32 && mw ? (int)threadIdx.x : lane;
+        // Two levels per pass: a lane's two units of level k are partners, so level k - 1 comes from
+        // them in registers instead of being read back (level 6 alone takes a pass when it is left).
+#pragma unroll 1
+        for (int k = min(t, n - 1); k >= 6;) {
+            const bool two = k > 6;
+            if (lead) {
+                const uint32_t both = two ? 3u << (k - 1) : 1u << k;
+                const uint32_t own = __reduce_or_sync(0xffffffffu, shA & both);
+#pragma unroll 1
+                for (int q = k; q >= k - (two ? 1 : 0); --q)
+                    if ((own >> q) & 1u) scl_own<W>(pA, q, act, L);
+                shA &= ~both;
             }
             const bool use_g = blk != 0 && k == t;
             const bool from_ch = k + 1 == n;
-            const int len = 1 << k;
-            float* dst = stage ? S.stage : S.A(k);
-            const int dstride = stage ? kSclStage : len;
+            const int len = 1 << k, sh = two ? k - 3 : k - 2;
+            float* dst = S.A(k);
+            float* dst2 = S.A(two ? k - 1 : k);
             const float* srcb = from_ch ? y : S.A(k + 1);
             const uint32_t* cbk = S.Cl(k);
-            const uint32_t my_d = stage ? (uint32_t)lane : fld(pA, k), my_s = from_ch ? 0u : fld(pA, k + 1),
-                           my_c = fld(pC, k);
+            // a path's arrays of levels k (written), k + 1 (read), of the partial sums of level k, and
+            // of level k - 1 (written)
+            const uint32_t mine = fld(pA, k) | (from_ch ? 0u : fld(pA, k + 1) << 8) | fld(pC, k) << 16 |
+                                  fld(pA, two ? k - 1 : k) << 24;
             int nact = act, nact_both = act_both;
-            if constexpr (MW) {
+            if constexpr (W == 32) {
                 if (lead) {
-                    ptab[lane] = my_d;
-                    ptab[32 + lane] = my_s;
-                    ptab[64 + lane] = my_c;
-                    if (lane == 0) ptab[96] = (uint32_t)act;
+                    ptab[lane] = mine;
+                    if (lane == 0) ptab[32] = (uint32_t)act;
                 }
-                __syncthreads();
-                nact = nact_both = (int)ptab[96];
+                level_sync();
+                nact = nact_both = (int)ptab[32];
             }
-            const int cwk = scl_cs(k);
-            // element stride of a round: the list's lanes, or every thread of the CTA
-            const int TW = MW ? (int)blockDim.x : W, tix = MW ? (int)threadIdx.x : lane;
-            // Units of four consecutive elements of one path (a level has at least 32): one 16-byte
-            // load per operand and one set of pointers per unit.  kSclUpRound units per lane per
-            // round: all loads of a round are issued before any store, so the L2 latency of the
-            // upper levels (global for long lists) is paid once per round.  The loads are
-            // unconditional (a unit past the list's end reads a valid slot: its path index is below
-            // L and its offset below len), so nothing but the stores is predicated and the rounds'
-            // independent chains interleave.
-            // CH: the level reads the channel row, whose values are staged as CA-SCL reads them;
-            // the caller's row may start at any float, so its 16-byte loads need `y16`.
-            auto rounds = [&](auto USE_G, auto FROM_CH) {
-                constexpr bool G = decltype(USE_G)::value, CH = decltype(FROM_CH)::value;
-                constexpr int U = kSclUpRound;
-                const int ku = k - 2, tot = nact << ku, tmax = nact_both << ku;
-                for (int e0 = 0; e0 < tmax; e0 += U * TW) {
-                    float4 va[U], vb[U];
-                    uint32_t vw[U], pdv[U];
+            const int cwk = scl_cs(k), tot = nact << sh, tmax = nact_both << sh;
+            // level 6 is stored with permuted chunks
+            const int swz = k == 6 ? 7 : 0, swz2 = k == 7 ? 7 : 0;
+            // Units of four consecutive elements of one path (a level has at least 64): one 16-byte
+            // load per operand and one set of pointers per unit, two units per lane and round.  All
+            // loads of a round are issued before any store, so the L2 latency of the upper levels
+            // (global for long lists) is paid once per round.  The loads are unconditional (a unit
+            // past the list's end reads a valid slot: its path index is below L and its offset below
+            // len), so nothing but the stores is predicated and the units' chains interleave.
+            // The channel row is staged as CA-SCL reads it; the caller's row may start at any float,
+            // so its 16-byte loads need `y16`.
+            auto rounds = [&](auto USE_G) {
+                constexpr bool G = decltype(USE_G)::value;
+#pragma unroll 1
+                for (int e0 = 0; e0 < tmax; e0 += two ? TW : 2 * TW) {
+                    float4 va[2], vb[2], r[2];
+                    uint32_t vw[2], ptr[2];
+                    int u[2];
 #pragma unroll
-                    for (int q = 0; q < U; ++q) {
-                        const int e = e0 + TW * q + tix;
-                        const int p = (e >> ku) & (W - 1);
-                        pdv[q] = MW ? ptab[p] : sg.shfl(my_d, p);
-                        const uint32_t ps = CH ? 0u : MW ? ptab[32 + p] : sg.shfl(my_s, p);
-                        const int j = (e << 2) & (len - 1);
-                        const float* src = srcb + ps * (2 * len) + j;
-                        if (CH && !y16) {
+                    for (int q = 0; q < 2; ++q) {
+                        const int e = e0 + tix + (two ? 0 : TW * q);
+                        const int p = (e >> sh) & (W - 1);
+                        u[q] = (e & ((1 << sh) - 1)) + (two ? q << sh : 0);
+                        ptr[q] = W == 32 ? ptab[p] : sg.shfl(mine, p);
+                        const float* src = srcb + ((((ptr[q] >> 8) & 31u) << (k + 1)) + 4 * u[q]);
+                        if (from_ch && !y16) {
                             va[q] = make_float4(src[0], src[1], src[2], src[3]);
                             vb[q] = make_float4(src[len], src[len + 1], src[len + 2], src[len + 3]);
                         } else {
@@ -607,84 +626,112 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                             vb[q] = *reinterpret_cast<const float4*>(src + len);
                         }
                         if constexpr (G)
-                            vw[q] = cbk[(MW ? ptab[64 + p] : sg.shfl(my_c, p)) * cwk + (j >> 5)] >> (j & 31);
+                            vw[q] = cbk[((ptr[q] >> 16) & 31u) * cwk + (u[q] >> 3)] >> (4 * (u[q] & 7));
                     }
 #pragma unroll
-                    for (int q = 0; q < U; ++q) {
-                        const int e = e0 + TW * q + tix;
-                        const int j = (e << 2) & (len - 1);
-                        float4 x = va[q], y4 = vb[q], r;
-                        if constexpr (CH) {
+                    for (int q = 0; q < 2; ++q) {
+                        const int d = ptr[q] & 31u;
+                        float4 x = va[q], y4 = vb[q];
+                        if (from_ch) {
                             x = make_float4(scl_stage(x.x), scl_stage(x.y), scl_stage(x.z), scl_stage(x.w));
                             y4 = make_float4(scl_stage(y4.x), scl_stage(y4.y), scl_stage(y4.z), scl_stage(y4.w));
                         }
                         if constexpr (G)
-                            r = make_float4(scl_g(x.x, y4.x, vw[q] & 1u), scl_g(x.y, y4.y, vw[q] & 2u),
-                                            scl_g(x.z, y4.z, vw[q] & 4u), scl_g(x.w, y4.w, vw[q] & 8u));
+                            r[q] = make_float4(scl_g(x.x, y4.x, vw[q], 0), scl_g(x.y, y4.y, vw[q], 1),
+                                               scl_g(x.z, y4.z, vw[q], 2), scl_g(x.w, y4.w, vw[q], 3));
                         else
-                            r = make_float4(xmin(x.x, y4.x), xmin(x.y, y4.y), xmin(x.z, y4.z), xmin(x.w, y4.w));
-                        if (e < tot) {
-                            float* d = dst + pdv[q] * dstride + j;
-                            if (stage) {  // staging rows have an odd stride
-                                d[0] = r.x;
-                                d[1] = r.y;
-                                d[2] = r.z;
-                                d[3] = r.w;
-                            } else {
-                                *reinterpret_cast<float4*>(d) = r;
-                            }
-                        }
+                            r[q] = make_float4(xmin(x.x, y4.x), xmin(x.y, y4.y), xmin(x.z, y4.z), xmin(x.w, y4.w));
+                        if (e0 + tix + (two ? 0 : TW * q) < tot)
+                            *reinterpret_cast<float4*>(dst + (d << k) + 4 * (u[q] ^ (d & swz))) = r[q];
+                    }
+                    if (two && e0 + tix < tot) {
+                        const int d = ptr[0] >> 24;
+                        *reinterpret_cast<float4*>(dst2 + (d << (k - 1)) + 4 * (u[0] ^ (d & swz2))) =
+                            make_float4(xmin(r[0].x, r[1].x), xmin(r[0].y, r[1].y), xmin(r[0].z, r[1].z),
+                                        xmin(r[0].w, r[1].w));
                     }
                 }
             };
-            if (from_ch) {
-                if (use_g)
-                    rounds(std::true_type{}, std::true_type{});
-                else
-                    rounds(std::false_type{}, std::true_type{});
-            } else if (use_g) {
-                rounds(std::true_type{}, std::false_type{});
-            } else {
-                rounds(std::false_type{}, std::false_type{});
-            }
-            if constexpr (MW)
-                __syncthreads();
+            if (use_g)
+                rounds(std::true_type{});
             else
-                __syncwarp();
+                rounds(std::false_type{});
+            level_sync();
+            k -= two ? 2 : 1;
         }
         if (!lead) continue;  // the helper warps only share the upper levels
         // ------------------------------------------------ the 32 bits of the block
         // A runtime walk of the block's tree, four bits at a time; one copy of the list step serves
         // all bits (unrolling it per bit overflowed the instruction cache).  Lanes past the list
-        // read row 0 (the staging area has L rows) and compute values nobody reads.
+        // work on its first array and row and compute values nobody reads.
         const uint32_t fw = C.frozen_bits[blk], dw = C.decided_bits[blk];
         uint32_t v5 = 0u;
         lf.row = lane < L ? lane : 0;
         int r = 0, failed = -1;  // failed: bit at which the full-list shortcut is known to fail
-        if (fw == 0u) {
-            const float* row = S.stage + lf.row * kSclStage;
-            if (leaf_all_hard<W, 32>(sg, [&](int j) { return row[j]; }, pm, act, L, v5)) r = 32;
-            else failed = 0;
+        {
+            // level 5 of this lane's path, from its level-6 array
+            float l5[32];
+            const int m6 = lane < L ? (int)fld(pA, 6) : 0;
+            const float* row6 = S.sA + m6 * 64;
+            const uint32_t c5 = S.Cl(5)[fld(pC, 5)];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const float4 x = *reinterpret_cast<const float4*>(row6 + scl_chunk(m6, c));
+                const float4 z = *reinterpret_cast<const float4*>(row6 + scl_chunk(m6, c + 8));
+                if (t == 5) {
+                    l5[4 * c] = scl_g(x.x, z.x, c5, 4 * c);
+                    l5[4 * c + 1] = scl_g(x.y, z.y, c5, 4 * c + 1);
+                    l5[4 * c + 2] = scl_g(x.z, z.z, c5, 4 * c + 2);
+                    l5[4 * c + 3] = scl_g(x.w, z.w, c5, 4 * c + 3);
+                } else {
+                    l5[4 * c] = xmin(x.x, z.x);
+                    l5[4 * c + 1] = xmin(x.y, z.y);
+                    l5[4 * c + 2] = xmin(x.z, z.z);
+                    l5[4 * c + 3] = xmin(x.w, z.w);
+                }
+            }
+            if (fw == 0u) {
+                if (leaf_all_hard(sg, l5, pm, act, L, v5))
+                    r = 32;
+                else
+                    failed = 0;
+            }
+            if (r == 0) {
+                if (lane < L) {
+                    float* row = S.stage + lane * kSclStage;
+#pragma unroll
+                    for (int c = 0; c < 8; ++c)
+                        *reinterpret_cast<float4*>(row + scl_chunk(lane, c)) =
+                            make_float4(l5[4 * c], l5[4 * c + 1], l5[4 * c + 2], l5[4 * c + 3]);
+                }
+#pragma unroll
+                for (int j = 0; j < 16; ++j) lf.l4[j] = xmin(l5[j], l5[j + 16]);
+                __syncwarp();
+            }
         }
 #pragma unroll 1
         while (r < 32) {
             uint32_t v = 0u;
             int k = 5;  // level of the node decided by this step; 5: none yet
             if ((r & 15) == 0) {
-                const float* row = S.stage + lf.row * kSclStage;
-                if (r == 0) {
+                if (r != 0) {
+                    const float* row = S.stage + lf.row * kSclStage;
 #pragma unroll
-                    for (int j = 0; j < 16; ++j) lf.l4[j] = xmin(row[j], row[j + 16]);
-                } else {
-#pragma unroll
-                    for (int j = 0; j < 16; ++j) lf.l4[j] = scl_g(row[j], row[j + 16], lf.c[4] & (1u << j));
+                    for (int c = 0; c < 4; ++c) {
+                        const float4 x = *reinterpret_cast<const float4*>(row + scl_chunk(lf.row, c));
+                        const float4 z = *reinterpret_cast<const float4*>(row + scl_chunk(lf.row, c + 4));
+                        lf.l4[4 * c] = scl_g(x.x, z.x, lf.c[4], 4 * c);
+                        lf.l4[4 * c + 1] = scl_g(x.y, z.y, lf.c[4], 4 * c + 1);
+                        lf.l4[4 * c + 2] = scl_g(x.z, z.z, lf.c[4], 4 * c + 2);
+                        lf.l4[4 * c + 3] = scl_g(x.w, z.w, lf.c[4], 4 * c + 3);
+                    }
                 }
                 const uint32_t f = (fw >> r) & 0xffffu;
                 if (f == 0xffffu) {
                     leaf_frozen(lf.l4, pm);
                     k = 4;
                 } else if (f == 0u && failed != r) {
-                    if (leaf_all_hard<W, 16>(sg, [&](int j) { return lf.l4[j]; }, pm, act, L, v)) k = 4;
+                    if (leaf_all_hard(sg, lf.l4, pm, act, L, v)) k = 4;
                     else failed = r;
                 }
             }
@@ -698,7 +745,7 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                     leaf_frozen(lf.l3, pm);
                     k = 3;
                 } else if (f == 0u && failed != r) {
-                    if (leaf_all_hard<W, 8>(sg, [&](int j) { return lf.l3[j]; }, pm, act, L, v)) k = 3;
+                    if (leaf_all_hard(sg, lf.l3, pm, act, L, v)) k = 3;
                     else failed = r;
                 }
             }
@@ -714,7 +761,7 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                     leaf_frozen(lf.l2, pm);
                     whole = true;
                 } else if (f == 0u && failed != r) {
-                    whole = leaf_all_hard<W, 4>(sg, [&](int j) { return lf.l2[j]; }, pm, act, L, v);
+                    whole = leaf_all_hard(sg, lf.l2, pm, act, L, v);
                     if (!whole) failed = r;
                 }
                 if (!whole) {
@@ -723,7 +770,7 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                     for (int q = r; q < r + 4; ++q) {
                         float lam;
                         if (q & 1) {
-                            lam = scl_g(lf.l1[0], lf.l1[1], lf.c[0] & 1u);
+                            lam = scl_g(lf.l1[0], lf.l1[1], lf.c[0], 0);
                         } else {
                             if (q & 2)
                                 leaf_g<2>(lf.l2, lf.l1, lf.c[1]);
@@ -867,21 +914,18 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
     }
     if (!lead) return;
     // ------------------------------------------------------------------ CRC selection
-    // The paths in (metric, index) order: the codeword x of each (its level-n array; the list's
-    // lanes hold the 32-bit words lane + W h) is turned into u = x G and its CRC syndrome, the XOR
-    // of the syndrome columns of the positions decided 1, is formed with one column per lane.  The
-    // first path whose syndrome is zero is output, the best one if none is.  On most frames that is
-    // one path's work, against a column load and XOR per path and bit, and a shuffle per list step,
-    // for syndromes kept along the way.
-    constexpr int H = kMaxWords / W;  // words per lane
+    // The paths in (metric, index) order: the codeword x of each (its level-n array) is turned into
+    // u = x G in place, and its CRC syndrome, the XOR of the syndrome columns of the positions
+    // decided 1, is formed with one column per lane.  The first path whose syndrome is zero is
+    // output, the best one if none is.  On most frames that is one path's work, against a column
+    // load and XOR per path and bit, and a shuffle per list step, for syndromes kept along the way.
     const int words = N >> 5;
     uint32_t* xl = S.Cl(n);
     const uint32_t my_x = fld(pC, n);
-    const uint32_t m[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
-    uint32_t best[H];   // u of the output path,
-    uint32_t* uw = xl;  // written back over its codeword, where the payload bits are picked from
-    bool avail = lane < act, done = act == 0, any_ok = false, first = true;
+    uint32_t* uw = nullptr;  // u of the output path
+    bool avail = lane < act, done = act == 0, any_ok = false;
     __syncwarp();
+#pragma unroll 1
     while (__any_sync(0xffffffffu, !done)) {
         float key = avail ? pm : __int_as_float(0x7f800000);
         int who = avail ? lane : 64;
@@ -895,59 +939,48 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
             }
         }
         uint32_t* xw = xl + sg.shfl(my_x, who & (W - 1)) * scl_cs(n);
-        uint32_t w[H];
+        uint32_t syn = 0u;
+        const bool on = !done;
+        if (on) {
+            const uint32_t m[5] = {0x55555555u, 0x33333333u, 0x0F0F0F0Fu, 0x00FF00FFu, 0x0000FFFFu};
+#pragma unroll 1
+            for (int i = lane; i < words; i += W) {
+                uint32_t x = xw[i];
 #pragma unroll
-        for (int h = 0; h < H; ++h) w[h] = (frame >= 0 && lane + W * h < words) ? xw[lane + W * h] : 0u;
-#pragma unroll
-        for (int h = 0; h < H; ++h)
-#pragma unroll
-            for (int e = 0; e < 5; ++e) w[h] ^= (w[h] >> (1 << e)) & m[e];
-        for (int D = 1; D < W && D < words; D <<= 1) {
-#pragma unroll
-            for (int h = 0; h < H; ++h) {
-                const uint32_t o = __shfl_xor_sync(0xffffffffu, w[h], D);
-                if (!(lane & D)) w[h] ^= o;
+                for (int e = 0; e < 5; ++e) x ^= (x >> (1 << e)) & m[e];
+                xw[i] = x;
             }
         }
-        for (int D = W; D < words; D <<= 1) {
-            const int hd = D / W;
-#pragma unroll
-            for (int h = 0; h < H; ++h)
-                if (!(h & hd) && (h | hd) < H) w[h] ^= w[h | hd];
+#pragma unroll 1
+        for (int D = 1; D < words; D <<= 1) {
+            __syncwarp();
+            if (on) {
+#pragma unroll 1
+                for (int i = lane; i < words >> 1; i += W) {  // word pair (j, j + D), bit log2 D of j clear
+                    const int j = ((i & ~(D - 1)) << 1) | (i & (D - 1));
+                    xw[j] ^= xw[j + D];
+                }
+            }
         }
-        uint32_t syn = 0u;
-#pragma unroll
-        for (int h = 0; h < H; ++h) {
-            const int cnt = min(W, words - W * h);
-            const uint32_t* col = C.colsyn + W * h * 32 + lane;
+        __syncwarp();
+        if (on) {
 #pragma unroll 4
-            for (int i = 0; i < cnt; ++i) {
-                const uint32_t ui = sg.shfl(w[h], i);
+            for (int i = 0; i < words; ++i) {
+                const uint32_t ui = xw[i];
 #pragma unroll
-                for (int z = 0; z < 32; z += W)
-                    if ((ui >> (lane + z)) & 1u) syn ^= col[32 * i + z];
+                for (int z = lane; z < 32 + lane; z += W)
+                    if ((ui >> z) & 1u) syn ^= C.colsyn[32 * i + z];
             }
         }
         syn = sg.red_xor(syn);
-        if (!done) {
+        if (on) {
             any_ok = syn == 0u;
-            if (first || any_ok) {
-#pragma unroll
-                for (int h = 0; h < H; ++h) best[h] = w[h];
-                uw = xw;
-            }
-            first = false;
+            if (!uw || any_ok) uw = xw;
             if (lane == who) avail = false;
         }
         const bool none_left = sg.ballot(avail) == 0u;
         done = done || any_ok || none_left;
     }
-    if (frame >= 0) {
-#pragma unroll
-        for (int h = 0; h < H; ++h)
-            if (lane + W * h < words) uw[lane + W * h] = best[h];
-    }
-    __syncwarp();
     if (frame >= 0) {
         uint8_t* out = a.bits + (size_t)frame * a.row_bytes;
         for (int by = lane; by < a.row_bytes; by += W) {
@@ -969,9 +1002,9 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
 // of a mixed batch (-1: the batch's single code): plan of the code, the list's shared words `ws`
 // and global slot `slot` (null: every level in shared memory).  A list without a frame still walks
 // the code's structure with no path, so both lists of a warp must be given the same code.
-template <bool TWO, int W, bool MW = false>
+template <bool TWO, int W>
 __device__ __forceinline__ void scl_warp_frame(const SCLArgs& a, int frame, int code_id, uint32_t* ws, float* slot,
-                                               uint8_t* selc, uint32_t* ptab = nullptr)
+                                               uint8_t* selc, uint32_t* ptab, bool mw)
 {
     constexpr int LISTS = 32 / W;
     const int L = a.L;
@@ -992,7 +1025,7 @@ __device__ __forceinline__ void scl_warp_frame(const SCLArgs& a, int frame, int 
     S.sC = reinterpret_cast<uint32_t*>(S.stage + L * kSclStage);
     S.gA = slot;
     S.gC = slot ? reinterpret_cast<uint32_t*>(slot + (size_t)L * (C.N - (2 << S.KS))) : nullptr;
-    scl_decode_frame<TWO, W, MW>(a, C, frame, S, selc, ptab);
+    scl_decode_frame<TWO, W>(a, C, frame, S, selc, ptab, mw);
 }
 
 // W = 32: one frame per warp; W = 16: two (one per half-warp list), claimed together.  In a mixed
@@ -1003,41 +1036,34 @@ __global__ void __launch_bounds__(kSclWarpsPerCTA * 32, 4) scl_kernel(const SCLA
 {
     constexpr int LISTS = 32 / W;
     extern __shared__ __align__(16) uint32_t smem[];
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const int li = lane / W;  // this lane's list
+    const int lane = threadIdx.x & 31, li = lane / W;  // this lane's list
+    const int count = a.count ? *a.count : a.B;
+    // Few frames (at most one per CTA, single code, whole-warp lists): each CTA takes one frame at a
+    // time and all its warps share the frame's upper-level updates, which shortens the frame's decoding
+    // latency: warp 0's list words, scratch and global slot serve the CTA's frame.
+    const bool mw = W == 32 && !a.code_of && count <= (int)gridDim.x && blockDim.x >= 64;
+    const int wid = mw ? 0 : threadIdx.x >> 5;
     uint32_t* wsw = smem + (size_t)wid * a.warp_words;
     uint32_t* ws = wsw + li * a.list_words;
-    uint8_t* selc = reinterpret_cast<uint8_t*>(wsw + a.warp_words - 16);
+    uint32_t* scratch = wsw + a.warp_words - kSclWarpWords;
+    uint8_t* selc = reinterpret_cast<uint8_t*>(scratch);
+    uint32_t* ptab = scratch + kSclScratch;
     float* slot = a.scratch
         ? a.scratch + (((size_t)blockIdx.x * (blockDim.x >> 5) + wid) * LISTS + li) * (size_t)a.slot_words
         : nullptr;
-    const int count = a.count ? *a.count : a.B;
-    if constexpr (W == 32) {
-        // Few frames (at most one per CTA, single code): each CTA takes one frame at a time and
-        // all its warps share the frame's upper-level updates (the words of warp 1, unused here,
-        // hold the shared path pointers), which shortens the frame's decoding latency.
-        if (!a.code_of && count <= (int)gridDim.x && blockDim.x >= 64) {
-            uint32_t* ptab = smem + a.warp_words;
-            // warp 0's list words, list-step scratch and global slot serve the CTA's frame
-            float* slot0 = a.scratch ? a.scratch + (size_t)blockIdx.x * (blockDim.x >> 5) * (size_t)a.slot_words : nullptr;
-            uint8_t* selc0 = reinterpret_cast<uint8_t*>(smem + a.warp_words - 16);
-            for (;;) {
-                if (threadIdx.x == 0) ptab[100] = (uint32_t)atomicAdd(a.next, 1);
-                __syncthreads();
-                const int idx = (int)ptab[100];
-                __syncthreads();
-                if (idx >= count) break;  // uniform over the CTA
-                scl_warp_frame<TWO, W, true>(a, a.list ? a.list[idx] : idx, -1, smem, slot0, selc0, ptab);
-                __syncthreads();
-            }
-            return;
-        }
-    }
+#pragma unroll 1
     for (;;) {
         int idx = 0;
-        if (lane == 0) idx = atomicAdd(a.next, LISTS);
-        idx = __shfl_sync(0xffffffffu, idx, 0);
-        if (idx >= count) break;  // uniform over the warp
+        if (mw) {
+            if (threadIdx.x == 0) ptab[33] = (uint32_t)atomicAdd(a.next, 1);
+            __syncthreads();
+            idx = (int)ptab[33];
+            __syncthreads();
+        } else {
+            if (lane == 0) idx = atomicAdd(a.next, LISTS);
+            idx = __shfl_sync(0xffffffffu, idx, 0);
+        }
+        if (idx >= count) break;  // uniform over the warp (mw: the CTA)
         const int k = idx + li;
         const int frame = k < count ? (a.list ? a.list[k] : k) : -1;
         // one call site: every inlined copy of the decoder would be scheduled and allocated apart
@@ -1053,21 +1079,22 @@ __global__ void __launch_bounds__(kSclWarpsPerCTA * 32, 4) scl_kernel(const SCLA
         }
 #pragma unroll 1
         for (int q = 0; q < passes; ++q)
-            scl_warp_frame<TWO, W>(a, passes == 1 || li == q ? frame : -1, q ? other : code, ws, slot, selc);
+            scl_warp_frame<TWO, W>(a, passes == 1 || li == q ? frame : -1, q ? other : code, ws, slot, selc, ptab, mw);
+        if (mw) __syncthreads();
     }
 }
 
 // Persistent launch: as many CTAs as fit on the device (bounded by the global slots and, when it
 // is known on the host, by the work); returns cudaSuccess or the launch error.
-cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int warp_words_max, long long slot_words_max)
+cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int list_words_max, long long slot_words_max)
 {
     const bool all_smem = a.scratch == nullptr;
     const int lists = scl_two_lists(L, all_smem) ? 2 : 1;
     const SCLPlan p = scl_plan(N, L, all_smem, lists);
     a.KS = p.KS;
     a.KC = p.KC;
-    a.list_words = std::max(p.list_words, warp_words_max - 16);
-    a.warp_words = lists * a.list_words + 16;
+    a.list_words = std::max(p.list_words, list_words_max);
+    a.warp_words = lists * a.list_words + kSclWarpWords;
     // slots hold 16-byte vectors: each starts on a 16-byte boundary, wherever the caller's workspace
     // starts, so the same scratch bytes may give a few slots less than it was sized for
     const long long slot_words = std::max(p.slot_words, slot_words_max);
