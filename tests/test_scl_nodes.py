@@ -51,12 +51,15 @@ def rows(ocode, B, seed, ties):
 @pytest.mark.parametrize("which,ties", [("nodes", False), ("nodes", True), ("decided", False), ("short", True)])
 def test_whole_nodes_bit_exact(which, ties, L):
     ocode = fr.oracle_code(128, 64, 8) if which == "short" else node_code(which == "decided")
-    B, N = 21, ocode.N
-    llr = rows(ocode, B, 500 + L, ties)
-    ref = oracle.scl_decode(llr, ocode, L, "f32")
+    N = ocode.N
+    some = rows(ocode, 21, 500 + L, ties)
+    ref = oracle.scl_decode(some, ocode, L, "f32")
     code = api.PolarCode(N, ocode.K, ocode.crc_len, ocode.frozen.copy(), ocode.crc_poly, decided=ocode.decided)
-    need = api.polar_workspace_bytes(code, B, L, api.POLAR_OP_SCL)
-    for skip in (0, 1):  # rows and workspace on and off a 16-byte boundary
+    # rows and workspace on and off a 16-byte boundary, few frames (a CTA each) and more than any grid
+    # has CTAs (a warp each, or two per warp)
+    for skip, times in ((0, 1), (1, 1), (1, 60)):
+        llr, B = np.tile(some, (times, 1)), 21 * times
+        need = api.polar_workspace_bytes(code, B, L, api.POLAR_OP_SCL)
         flat = torch.empty(B * N + 4, dtype=torch.float32, device="cuda")
         x = flat[skip:skip + B * N].view(B, N)
         x.copy_(torch.from_numpy(llr))
@@ -65,5 +68,6 @@ def test_whole_nodes_bit_exact(which, ties, L):
         status = torch.zeros(B, dtype=torch.uint8, device="cuda")
         api.scl_decode(code, x, L, bits, status, ws)
         torch.cuda.synchronize()
-        assert np.array_equal(status.cpu().numpy(), ref["status"])
-        assert np.array_equal(api.unpack_bits(bits.cpu().numpy(), code.P), oracle.payload_of(ref["u_hat"], ocode))
+        assert np.array_equal(status.cpu().numpy(), np.tile(ref["status"], times))
+        assert np.array_equal(api.unpack_bits(bits.cpu().numpy(), code.P),
+                              np.tile(oracle.payload_of(ref["u_hat"], ocode), (times, 1)))
