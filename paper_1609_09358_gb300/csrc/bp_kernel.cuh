@@ -415,18 +415,22 @@ struct BPKernelPlan<10, 0, 0, FPT> {
     static constexpr int F = 1;
 };
 template <>
+struct BPKernelPlan<10, 0, 4, 1> : BPKernelPlan<10, 0, 0, 1> {};
+template <>
 struct BPKernelPlan<12, 0, 0, 1> {
     using Plan = BPPlan<12, 4>;
     static constexpr int F = 1;
 };
 
-template <class P>
+template <class P, bool CYC = false>
 __host__ __device__ constexpr int bp_slot_words()
 {
     // exchange buffers [2][XW] | syndrome columns, thread-major [R][T] | partial syndromes
-    // [2][2][NW] | packed payload bits [2][N/32] | fetched frame index [4] | from N = 1024 on the
-    // channel column [XW], in the last group's exchange layout
-    return 2 * P::XW + P::N + 4 * P::NW + 2 * (P::N / 32) + 4 + (P::LOGN >= 10 ? P::XW : 0);
+    // [2][2][NW] | packed payload bits [2][N/32] | fetched frame index [4] | from
+    // N = 1024 on the channel column [XW], in the last group's exchange layout | CYC: saved L columns
+    // 2..n [n-1][R][T]
+    return 2 * P::XW + P::N + 4 * P::NW + 2 * (P::N / 32) + 4 + (P::LOGN >= 10 ? P::XW : 0) +
+           (CYC ? (P::LOGN - 1) * P::N : 0);
 }
 
 // One frame group of T threads decoding frames from `src` until it runs dry.  Group `slot` of
@@ -435,7 +439,8 @@ __host__ __device__ constexpr int bp_slot_words()
 // the PE pairs keeps the syndrome columns of two adjacent nodes in one word.
 // VAR (FP32, unweighted): bit 0 the exact PE function instead of min-sum, bit 1 the re-encoding
 // stop -- the frame stops at the first iteration where HD(LLR(x)) equals the re-encoded HD(LLR(u))
-// (x = u G, Sec. II-B) and counts as decoded iff its CRC then holds.
+// (x = u G, Sec. II-B) and counts as decoded iff its CRC then holds; bit 2 (alone) min-sum with skipped
+// periods of repeating frames (CYC below): the same results as VAR 0.
 template <int R>
 __host__ __device__ constexpr uint32_t pe_low_mask(int dd)
 {
@@ -511,6 +516,23 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     int xbase[NG];                                         // exchange base of each group (PAD plans)
     static_for<0, NG>([&](auto G) { xbase[G.value] = P::addr(P::tpart(G.value, t)); });
     uint32_t* synp = csyn + N;                             // [2 parity][2 frame][NW]
+    // CYC: min-sum BP without learned scales is a deterministic map of the messages an iteration hands
+    // to the next, so once they recur the frame repeats itself: no later iteration gives a hard decision
+    // that an earlier one of the period has not given, and the state after max_iters is known.  Of the
+    // frames that fail at N = 1024, K = 512, 2.5 dB about half end in a period of 1, 2 or 4 iterations,
+    // half of them within 20, and they took a sixth of all frame-iterations (a failing frame runs to
+    // max_iters = 200).  Every fourth iteration the syndrome is compared with the one four before;
+    // equal twice in a row is the cue: the messages are saved, compared bit by bit four iterations
+    // later, and if all are equal the iteration count moves on by the largest multiple of 4 that does
+    // not pass max_iters.  Everything written out is what the skipped iterations would have given.
+    // This happens where the stop decision already parts the iteration (DEFER): the messages that
+    // matter there are the columns R[2..SC+1] of the sweep under way (the last one in the exchange
+    // buffer) and L[SC+2..n].  At the loop's start, where they would be L[2..n], the extra branch kept
+    // the compiler from overlapping the syndrome with the next sweep and cost 10% of every iteration;
+    // here the kernel's iterations are 7% longer than the plain one's (launch_bp chooses).
+    // Measured: the production hybrid (N = 1024, K = 512, 10^5 frames, 2.5 dB) 4.33 -> 3.91 ms.
+    constexpr bool CYC = (VAR & 4) != 0;
+    static_assert(!CYC || (VAR == 4 && T > 32 && std::is_same<Src, CounterSource>::value), "repeats: plain FP32 min-sum");
     uint32_t* pbits = synp + 4 * NW;                       // [2 frame][N/32]
     int* fetched = reinterpret_cast<int*>(pbits + 2 * (N / 32));
     // CHS (N >= 1024): the channel column lives in shared memory and is read into registers at the
@@ -521,6 +543,10 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     // aligned-pair half2 kernels at N = 1024 (3.4% and 0.2% slower with it).
     constexpr bool CHS = n >= 11 || (n == 10 && (FPT == 1 || WEIGHTED == 1));
     MSG* chs = reinterpret_cast<MSG*>(fetched + 4);
+    uint32_t* saved = reinterpret_cast<uint32_t*>(fetched + 4 + (n >= 10 ? P::XW : 0));
+    int cue = 0;  // equal syndromes in a row (negative: looks to wait after a miss)
+    bool is_saved = false;
+    uint32_t last_syn = 0;
 
     // Frames of this group: half h (h < FPT) decodes frame fr[h]; when it stops it fetches the
     // next frame from the source.
@@ -718,73 +744,182 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                            !(EXACT && n == 12) && std::is_same<Src, CounterSource>::value;
     bool pending = false;  // DEFER: an iteration's partial syndromes are written, not yet read
     int it = 0;  // iterations run by this group (selects the partial-syndrome slot parity)
-    for (;;) {
-        // scales of the stage being computed and of the next one (loaded a stage ahead)
-        WSet wc{}, wn{};
-        if constexpr (WEIGHTED) wc = wload(0, 1);
-        uint32_t xh = 0;  // re-encoding stop: HD(LLR(x)) of this thread's channel-column nodes
-        // ------------------------------------------------------------------ R sweep
-        auto rstage = [&](auto S) {
-            constexpr int s = S.value, q = s - 1, g = P::grp(q), dd = 1 << (q - P::win(g));
-            constexpr bool last = s == n;
-            constexpr bool cross = P::rcross(s);
-            MSG* xb = xbuf + (P::xidx_r(s) & 1) * P::XW;
-            if constexpr (WEIGHTED) wn = last ? wload(1, n) : wload(0, s + 1);
-            if constexpr (last) chan_reload();
-            // outputs of the PE (k, k2): R[s+1] registers, the exchange buffer, or (last stage) only
-            // the re-encoding stop's hard decisions of LLR(x)
-            auto emit = [&](int k, int k2, MSG o1, MSG o2) {
-                if constexpr (REENC && last) {
-                    // LLR(x) = L[n+1] + R[n+1]: the channel column plus this stage's output
-                    xh |= (MT::neg(fadd(Lc[s + 1][k], o1), 0) ? 1u : 0u) << k;
-                    xh |= (MT::neg(fadd(Lc[s + 1][k2], o2), 0) ? 1u : 0u) << k2;
+    // scales of the stage being computed and of the next one (loaded a stage ahead)
+    WSet wc{}, wn{};
+    uint32_t xh = 0;              // re-encoding stop: HD(LLR(x)) of this thread's channel-column nodes
+    uint32_t syn0 = 0, syn1 = 0;  // this thread's part of the iteration's syndromes
+    // ---------------------------------------------------------------------- stages of the R sweep
+    auto rstage = [&](auto S) {
+        constexpr int s = S.value, q = s - 1, g = P::grp(q), dd = 1 << (q - P::win(g));
+        constexpr bool last = s == n;
+        constexpr bool cross = P::rcross(s);
+        MSG* xb = xbuf + (P::xidx_r(s) & 1) * P::XW;
+        if constexpr (WEIGHTED) wn = last ? wload(1, n) : wload(0, s + 1);
+        if constexpr (last) chan_reload();
+        // outputs of the PE (k, k2): R[s+1] registers, the exchange buffer, or (last stage) only
+        // the re-encoding stop's hard decisions of LLR(x)
+        auto emit = [&](int k, int k2, MSG o1, MSG o2) {
+            if constexpr (REENC && last) {
+                // LLR(x) = L[n+1] + R[n+1]: the channel column plus this stage's output
+                xh |= (MT::neg(fadd(Lc[s + 1][k], o1), 0) ? 1u : 0u) << k;
+                xh |= (MT::neg(fadd(Lc[s + 1][k2], o2), 0) ? 1u : 0u) << k2;
+            }
+            if constexpr (!last) {
+                if constexpr (cross) {
+                    xput<P, g>(xb, xbase, t, k, o1);
+                    xput<P, g>(xb, xbase, t, k2, o2);
+                } else {
+                    Rc[s + 1][k] = o1;
+                    Rc[s + 1][k2] = o2;
                 }
-                if constexpr (!last) {
-                    if constexpr (cross) {
-                        xput<P, g>(xb, xbase, t, k, o1);
-                        xput<P, g>(xb, xbase, t, k2, o2);
-                    } else {
-                        Rc[s + 1][k] = o1;
-                        Rc[s + 1][k2] = o2;
-                    }
-                }
-            };
-            if constexpr (PAIRS) {
+            }
+        };
+        if constexpr (PAIRS) {
 #pragma unroll
-                for (int i = 0; i < R / 2; i += 2) {
-                    const int kA = pe_k(dd, i), kB = pe_k(dd, i + 1), kA2 = kA | dd, kB2 = kB | dd;
-                    const float2 a1 = make_float2(Rc[s][kA], Rc[s][kB]);
-                    const float2 a2 = make_float2(Rc[s][kA2], Rc[s][kB2]);
-                    const float2 o1 = gpair(a1, __fadd2_rn(make_float2(Lc[s + 1][kA2], Lc[s + 1][kB2]), a2));
-                    const float2 o2 = __fadd2_rn(gpair(a1, make_float2(Lc[s + 1][kA], Lc[s + 1][kB])), a2);
-                    emit(kA, kA2, o1.x, clipm(o2.x, M));
-                    emit(kB, kB2, o1.y, clipm(o2.y, M));
+            for (int i = 0; i < R / 2; i += 2) {
+                const int kA = pe_k(dd, i), kB = pe_k(dd, i + 1), kA2 = kA | dd, kB2 = kB | dd;
+                const float2 a1 = make_float2(Rc[s][kA], Rc[s][kB]);
+                const float2 a2 = make_float2(Rc[s][kA2], Rc[s][kB2]);
+                const float2 o1 = gpair(a1, __fadd2_rn(make_float2(Lc[s + 1][kA2], Lc[s + 1][kB2]), a2));
+                const float2 o2 = __fadd2_rn(gpair(a1, make_float2(Lc[s + 1][kA], Lc[s + 1][kB])), a2);
+                emit(kA, kA2, o1.x, clipm(o2.x, M));
+                emit(kB, kB2, o1.y, clipm(o2.y, M));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                if (k & dd) continue;
+                const int k2 = k | dd;
+                const MSG a1 = Rc[s][k], a2 = Rc[s][k2], l1 = Lc[s + 1][k], l2 = Lc[s + 1][k2];
+                MSG o1, gg;
+                gf2(a1, fadd(l2, a2), a1, l1, o1, gg);
+                if constexpr (WEIGHTED) {
+                    o1 = fmul(wk(wc, k), o1);
+                    if constexpr (!UNIT) o1 = clipm(o1, Mv);
+                    gg = fmul(wk(wc, k2), gg);
+                }
+                emit(k, k2, o1, clipm(fadd(gg, a2), Mv));
+            }
+        }
+        if constexpr (cross) {
+            group_sync<T, SHARED_CTA>(slot);
+            if constexpr (!(DEFER && s == SC)) {
+#pragma unroll
+                for (int k = 0; k < R; ++k) Rc[s + 1][k] = xget<P, P::grp(s)>(xb, xbase, t, k);
+            }
+        }
+        if constexpr (WEIGHTED) wc = wn;
+    };
+    // ---------------------------------------------------------------------- stages of the L sweep
+    auto lstage = [&](auto S) {
+        constexpr int s = S.value, q = s - 1, g = P::grp(q), dd = 1 << (q - P::win(g));
+        constexpr bool first = s == 1;
+        constexpr bool cross = P::lcross(s);
+        MSG* xb = xbuf + (P::xidx_l(s) & 1) * P::XW;
+        if constexpr (WEIGHTED && !first) wn = wload(1, s - 1);
+        if constexpr (s == n) chan_reload();
+        auto emit = [&](int k, int k2, MSG o1, MSG o2) {
+            if constexpr (cross) {
+                xput<P, g>(xb, xbase, t, k, o1);
+                xput<P, g>(xb, xbase, t, k2, o2);
+            } else {
+                Lc[s][k] = o1;
+                Lc[s][k2] = o2;
+            }
+        };
+        if constexpr (PAIRS) {
+#pragma unroll
+            for (int i = 0; i < R / 2; i += 2) {
+                const int kA = pe_k(dd, i), kB = pe_k(dd, i + 1), kA2 = kA | dd, kB2 = kB | dd;
+                const float2 l1 = make_float2(Lc[s + 1][kA], Lc[s + 1][kB]);
+                const float2 l2 = make_float2(Lc[s + 1][kA2], Lc[s + 1][kB2]);
+                const float2 o1 = gpair(l1, __fadd2_rn(l2, make_float2(Rc[s][kA2], Rc[s][kB2])));
+                const float2 o2 = __fadd2_rn(gpair(make_float2(Rc[s][kA], Rc[s][kB]), l1), l2);
+                emit(kA, kA2, o1.x, clipm(o2.x, M));
+                emit(kB, kB2, o1.y, clipm(o2.y, M));
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                if (k & dd) continue;
+                const int k2 = k | dd;
+                const MSG a1 = Rc[s][k], a2 = Rc[s][k2], l1 = Lc[s + 1][k], l2 = Lc[s + 1][k2];
+                MSG o1, gg;
+                gf2(l1, fadd(l2, a2), a1, l1, o1, gg);
+                if constexpr (WEIGHTED) {
+                    o1 = fmul(wk(wc, k), o1);
+                    if constexpr (!UNIT) o1 = clipm(o1, Mv);
+                    gg = fmul(wk(wc, k2), gg);
+                }
+                emit(k, k2, o1, clipm(fadd(gg, l2), Mv));
+            }
+        }
+        if constexpr (cross) {
+            group_sync<T, SHARED_CTA>(slot);
+#pragma unroll
+            for (int k = 0; k < R; ++k) Lc[s][k] = xget<P, P::grp(s - 2)>(xb, xbase, t, k);
+        }
+        if constexpr (WEIGHTED && !first) wc = wn;
+        if constexpr (first) {
+            // hard decision of LLR(u) = L[1] + R[1]; XOR of the syndrome columns of the
+            // information nodes decided 1 (frozen nodes have column 0).  On an information
+            // node R[1] = +0, so u is never -0 and its sign bit is exactly (u < 0): the
+            // decision is an arithmetic shift and the update one and-xor.
+            if constexpr (syn_nodes) {
+                // one byte permute replicates the sign bits of u[k] and u[k + 1] into a 16|16
+                // mask over the pair's column word; one 64-bit load brings two such words
+                const uint2* cs2 = reinterpret_cast<const uint2*>(csyn);
+#pragma unroll
+                for (int k = 0; k < R; k += 4) {
+                    const uint2 cw = cs2[(k >> 2) * T + t];
+                    const float2 u0 = __fadd2_rn(make_float2(Lc[1][k], Lc[1][k + 1]),
+                                                 make_float2(Rc[1][k], Rc[1][k + 1]));
+                    const float2 u1 = __fadd2_rn(make_float2(Lc[1][k + 2], Lc[1][k + 3]),
+                                                 make_float2(Rc[1][k + 2], Rc[1][k + 3]));
+                    uint32_t m0, m1;
+                    asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(m0) : "r"(__float_as_uint(u0.x)), "r"(__float_as_uint(u0.y)));
+                    asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(m1) : "r"(__float_as_uint(u1.x)), "r"(__float_as_uint(u1.y)));
+                    syn0 ^= cw.x & m0;
+                    syn0 ^= cw.y & m1;
+                }
+            } else if constexpr (syn_packed) {
+                // one byte permute replicates the sign bits of both halves into a 16|16 mask
+#pragma unroll
+                for (int k = 0; k < R; ++k) {
+                    const MSG u = fadd(Lc[1][k], Rc[1][k]);
+                    uint32_t ub, m;
+                    memcpy(&ub, &u, 4);
+                    asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(m) : "r"(ub));
+                    syn0 ^= csyn[k * T + t] & m;
+                }
+            } else if constexpr (PAIRS) {
+#pragma unroll
+                for (int k = 0; k < R; k += 2) {
+                    const float2 u = __fadd2_rn(make_float2(Lc[1][k], Lc[1][k + 1]),
+                                                make_float2(Rc[1][k], Rc[1][k + 1]));
+                    syn0 ^= csyn[k * T + t] & (uint32_t)(__float_as_int(u.x) >> 31);
+                    syn0 ^= csyn[(k + 1) * T + t] & (uint32_t)(__float_as_int(u.y) >> 31);
                 }
             } else {
 #pragma unroll
                 for (int k = 0; k < R; ++k) {
-                    if (k & dd) continue;
-                    const int k2 = k | dd;
-                    const MSG a1 = Rc[s][k], a2 = Rc[s][k2], l1 = Lc[s + 1][k], l2 = Lc[s + 1][k2];
-                    MSG o1, gg;
-                    gf2(a1, fadd(l2, a2), a1, l1, o1, gg);
-                    if constexpr (WEIGHTED) {
-                        o1 = fmul(wk(wc, k), o1);
-                        if constexpr (!UNIT) o1 = clipm(o1, Mv);
-                        gg = fmul(wk(wc, k2), gg);
+                    const MSG u = fadd(Lc[1][k], Rc[1][k]);
+                    const uint32_t col = csyn[k * T + t];
+                    uint32_t ub;
+                    memcpy(&ub, &u, 4);
+                    if constexpr (FPT == 2) {
+                        syn0 ^= col & (uint32_t)((int32_t)(ub << 16) >> 31);
+                        syn1 ^= col & (uint32_t)((int32_t)ub >> 31);
+                    } else {
+                        syn0 ^= col & (uint32_t)((int32_t)ub >> 31);
                     }
-                    emit(k, k2, o1, clipm(fadd(gg, a2), Mv));
                 }
             }
-            if constexpr (cross) {
-                group_sync<T, SHARED_CTA>(slot);
-                if constexpr (!(DEFER && s == SC)) {
-#pragma unroll
-                    for (int k = 0; k < R; ++k) Rc[s + 1][k] = xget<P, P::grp(s)>(xb, xbase, t, k);
-                }
-            }
-            if constexpr (WEIGHTED) wc = wn;
-        };
+        }
+    };
+    for (;;) {
+        xh = syn0 = syn1 = 0;
+        if constexpr (WEIGHTED) wc = wload(0, 1);
         if constexpr (DEFER) {
             static_for<1, SC + 1>(rstage);
             if (pending) {
@@ -796,11 +931,56 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                 for (int w = 0; w < NW; ++w) sy ^= sp[w];
                 if constexpr (syn_nodes) sy = (sy ^ (sy >> 16)) & 0xFFFFu;
                 const bool ok = sy == 0u;
-                if ((ok && !a.fixed_iters) || itc[0] >= a.max_iters) {
-                    finalize(0, itc[0], ok);
-                    refill(0);
-                    if (fr[0] < 0) break;
-                    continue;  // the new frame starts its first R sweep
+                bool stop = (ok && !a.fixed_iters) || itc[0] >= a.max_iters, look = false;
+                if constexpr (CYC) {
+                    // (selects, no branch: a jump to code outside the loop every fourth iteration waited
+                    // for its instructions, 3% of the iteration)
+                    const bool fourth = (itc[0] & 3) == 0;
+                    const int c1 = cue < 0 || sy == last_syn ? cue + 1 : 0;
+                    cue = fourth ? c1 : cue;
+                    last_syn = fourth ? sy : last_syn;
+                    look = fourth && cue >= 2;
+                    if (fourth && cue < 2) is_saved = false;
+                }
+                if (stop || look) {
+                    if constexpr (CYC) {
+                        if (!stop) {
+                            // column c - 2 of the saved state: R[c] up to SC + 1, L[c] beyond
+                            auto column = [&](int c, int k) -> uint32_t {
+                                return __float_as_uint(c <= SC ? Rc[c][k] : c == SC + 1
+                                                           ? xget<P, P::grp(SC)>(xbuf + (P::xidx_r(SC) & 1) * P::XW, xbase, t, k)
+                                                           : Lc[c][k]);
+                            };
+                            if (is_saved) {
+                                uint32_t diff = 0;
+#pragma unroll
+                                for (int c = 2; c <= n; ++c)
+#pragma unroll
+                                    for (int k = 0; k < R; ++k) diff |= saved[((c - 2) * R + k) * T + t] ^ column(c, k);
+                                is_saved = false;
+                                cue = -4;
+                                if (__syncthreads_and(diff == 0u)) {
+                                    // this iteration and the three before it, none of which stopped, repeat
+                                    itc[0] += (a.max_iters - itc[0]) & ~3;
+                                    stop = itc[0] >= a.max_iters;
+                                }
+                            } else {
+#pragma unroll
+                                for (int c = 2; c <= n; ++c)
+#pragma unroll
+                                    for (int k = 0; k < R; ++k) saved[((c - 2) * R + k) * T + t] = column(c, k);
+                                is_saved = true;
+                            }
+                        }
+                    }
+                    if (stop) {
+                        finalize(0, itc[0], ok);
+                        refill(0);
+                        cue = 0;
+                        is_saved = false;
+                        if (fr[0] < 0) break;
+                        continue;  // the new frame starts its first R sweep
+                    }
                 }
             }
 #pragma unroll
@@ -809,114 +989,7 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
         } else {
             static_for<1, n + 1>(rstage);
         }
-        // ------------------------------------------------------------------ L sweep
-        uint32_t syn0 = 0, syn1 = 0;
-        static_for_down<n, 1>([&](auto S) {
-            constexpr int s = S.value, q = s - 1, g = P::grp(q), dd = 1 << (q - P::win(g));
-            constexpr bool first = s == 1;
-            constexpr bool cross = P::lcross(s);
-            MSG* xb = xbuf + (P::xidx_l(s) & 1) * P::XW;
-            if constexpr (WEIGHTED && !first) wn = wload(1, s - 1);
-            if constexpr (s == n) chan_reload();
-            auto emit = [&](int k, int k2, MSG o1, MSG o2) {
-                if constexpr (cross) {
-                    xput<P, g>(xb, xbase, t, k, o1);
-                    xput<P, g>(xb, xbase, t, k2, o2);
-                } else {
-                    Lc[s][k] = o1;
-                    Lc[s][k2] = o2;
-                }
-            };
-            if constexpr (PAIRS) {
-#pragma unroll
-                for (int i = 0; i < R / 2; i += 2) {
-                    const int kA = pe_k(dd, i), kB = pe_k(dd, i + 1), kA2 = kA | dd, kB2 = kB | dd;
-                    const float2 l1 = make_float2(Lc[s + 1][kA], Lc[s + 1][kB]);
-                    const float2 l2 = make_float2(Lc[s + 1][kA2], Lc[s + 1][kB2]);
-                    const float2 o1 = gpair(l1, __fadd2_rn(l2, make_float2(Rc[s][kA2], Rc[s][kB2])));
-                    const float2 o2 = __fadd2_rn(gpair(make_float2(Rc[s][kA], Rc[s][kB]), l1), l2);
-                    emit(kA, kA2, o1.x, clipm(o2.x, M));
-                    emit(kB, kB2, o1.y, clipm(o2.y, M));
-                }
-            } else {
-#pragma unroll
-                for (int k = 0; k < R; ++k) {
-                    if (k & dd) continue;
-                    const int k2 = k | dd;
-                    const MSG a1 = Rc[s][k], a2 = Rc[s][k2], l1 = Lc[s + 1][k], l2 = Lc[s + 1][k2];
-                    MSG o1, gg;
-                    gf2(l1, fadd(l2, a2), a1, l1, o1, gg);
-                    if constexpr (WEIGHTED) {
-                        o1 = fmul(wk(wc, k), o1);
-                        if constexpr (!UNIT) o1 = clipm(o1, Mv);
-                        gg = fmul(wk(wc, k2), gg);
-                    }
-                    emit(k, k2, o1, clipm(fadd(gg, l2), Mv));
-                }
-            }
-            if constexpr (cross) {
-                group_sync<T, SHARED_CTA>(slot);
-#pragma unroll
-                for (int k = 0; k < R; ++k) Lc[s][k] = xget<P, P::grp(s - 2)>(xb, xbase, t, k);
-            }
-            if constexpr (WEIGHTED && !first) wc = wn;
-            if constexpr (first) {
-                // hard decision of LLR(u) = L[1] + R[1]; XOR of the syndrome columns of the
-                // information nodes decided 1 (frozen nodes have column 0).  On an information
-                // node R[1] = +0, so u is never -0 and its sign bit is exactly (u < 0): the
-                // decision is an arithmetic shift and the update one and-xor.
-                if constexpr (syn_nodes) {
-                    // one byte permute replicates the sign bits of u[k] and u[k + 1] into a 16|16
-                    // mask over the pair's column word; one 64-bit load brings two such words
-                    const uint2* cs2 = reinterpret_cast<const uint2*>(csyn);
-#pragma unroll
-                    for (int k = 0; k < R; k += 4) {
-                        const uint2 cw = cs2[(k >> 2) * T + t];
-                        const float2 u0 = __fadd2_rn(make_float2(Lc[1][k], Lc[1][k + 1]),
-                                                     make_float2(Rc[1][k], Rc[1][k + 1]));
-                        const float2 u1 = __fadd2_rn(make_float2(Lc[1][k + 2], Lc[1][k + 3]),
-                                                     make_float2(Rc[1][k + 2], Rc[1][k + 3]));
-                        uint32_t m0, m1;
-                        asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(m0) : "r"(__float_as_uint(u0.x)), "r"(__float_as_uint(u0.y)));
-                        asm("prmt.b32 %0, %1, %2, 0xFFBB;" : "=r"(m1) : "r"(__float_as_uint(u1.x)), "r"(__float_as_uint(u1.y)));
-                        syn0 ^= cw.x & m0;
-                        syn0 ^= cw.y & m1;
-                    }
-                } else if constexpr (syn_packed) {
-                    // one byte permute replicates the sign bits of both halves into a 16|16 mask
-#pragma unroll
-                    for (int k = 0; k < R; ++k) {
-                        const MSG u = fadd(Lc[1][k], Rc[1][k]);
-                        uint32_t ub, m;
-                        memcpy(&ub, &u, 4);
-                        asm("prmt.b32 %0, %1, 0, 0xBB99;" : "=r"(m) : "r"(ub));
-                        syn0 ^= csyn[k * T + t] & m;
-                    }
-                } else if constexpr (PAIRS) {
-#pragma unroll
-                    for (int k = 0; k < R; k += 2) {
-                        const float2 u = __fadd2_rn(make_float2(Lc[1][k], Lc[1][k + 1]),
-                                                    make_float2(Rc[1][k], Rc[1][k + 1]));
-                        syn0 ^= csyn[k * T + t] & (uint32_t)(__float_as_int(u.x) >> 31);
-                        syn0 ^= csyn[(k + 1) * T + t] & (uint32_t)(__float_as_int(u.y) >> 31);
-                    }
-                } else {
-#pragma unroll
-                    for (int k = 0; k < R; ++k) {
-                        const MSG u = fadd(Lc[1][k], Rc[1][k]);
-                        const uint32_t col = csyn[k * T + t];
-                        uint32_t ub;
-                        memcpy(&ub, &u, 4);
-                        if constexpr (FPT == 2) {
-                            syn0 ^= col & (uint32_t)((int32_t)(ub << 16) >> 31);
-                            syn1 ^= col & (uint32_t)((int32_t)ub >> 31);
-                        } else {
-                            syn0 ^= col & (uint32_t)((int32_t)ub >> 31);
-                        }
-                    }
-                }
-            }
-        });
+        static_for_down<n, 1>(lstage);
         // ------------------------------------------------------------------ CRC early stop
         syn0 = __reduce_xor_sync(0xffffffffu, syn0);
         if constexpr (DEFER) {
@@ -1044,8 +1117,8 @@ __global__ void __launch_bounds__(THREADS, bp_min_ctas<LOGN, WEIGHTED, VAR>()) b
     const int t = threadIdx.x % P::T;
     constexpr int FPT = MsgTraits<MSG>::FPT;
     CounterSource src{a.next, a.B, (int)((blockIdx.x * F + slot) * FPT), FPT, a.frame0};
-    bp_run_group<P, MSG, WEIGHTED, false, CounterSource, SYNP, VAR>(a, *a.code, slot, t,
-                                                                    smem + slot * bp_slot_words<P>(), src);
+    constexpr int words = bp_slot_words<P, (VAR & 4) != 0>();
+    bp_run_group<P, MSG, WEIGHTED, false, CounterSource, SYNP, VAR>(a, *a.code, slot, t, smem + slot * words, src);
 }
 
 }  // namespace polar

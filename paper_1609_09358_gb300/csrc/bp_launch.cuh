@@ -21,6 +21,8 @@ struct BPKernelInfo {
 BPKernelInfo bp_kernel_info_fp32(int logn, int weighted, bool packed_syndrome);
 // FP32 unweighted kernel of a BP variant: bit 0 exact PE function, bit 1 re-encoding stop
 BPKernelInfo bp_kernel_info_fp32_var(int logn, int var);
+// FP32 min-sum kernel that skips the periods of repeating frames (N = 1024), else a null function
+BPKernelInfo bp_kernel_info_fp32_cyc(int logn, bool packed_syndrome);
 BPKernelInfo bp_kernel_info_fp16(int logn, int weighted, bool packed_syndrome);
 // natural-layout learned weights [iters][2][n][N] -> the prepared layout of the length's plan
 cudaError_t wms_prepare_fp32(int logn, const float* w, int iters, void* out, cudaStream_t st);

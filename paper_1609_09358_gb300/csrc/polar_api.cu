@@ -342,6 +342,12 @@ static int bp_variant(int precision)
 }
 static int bp_message(int precision) { return precision & ~(POLAR_G_EXACT | POLAR_STOP_REENCODE | POLAR_WMS_UNIT); }
 
+// From these iteration limits and batch sizes on the FP32 min-sum kernel that recognises repeating frames
+// is taken (N = 1024): its iterations take 7% longer, and it needs about 25 to find a repetition, so it
+// pays only if failing frames would run on well beyond that and if other frames wait for their place (a
+// batch that is resident at once ends with its longest frame, and not every failing frame repeats).
+constexpr int kBPCycleIters = 48, kBPCycleFrames = 2048;
+
 static int launch_bp(const DevCode* dcode, const polar_code* code, const float* llr, int B, int max_iters,
                      float llr_max, int precision, const void* w, int w_iters, uint8_t* bits, uint8_t* status,
                      uint16_t* iters, float* llr_u, float* llr_x, int* fail_count, int* fail_list,
@@ -379,9 +385,13 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
     // learned scales: the half2 form with both frames of a register on the same iteration when
     // the caller vouches for scales within [-1, 1] and every iteration is a learned one
     const int weighted = !w ? 0 : (unit && precision == POLAR_FP16 && max_iters <= w_iters) ? 2 : 1;
-    const BPKernelInfo k = precision == POLAR_FP16 ? bp_kernel_info_fp16(n, weighted, code->crc_len <= 16)
+    BPKernelInfo k = precision == POLAR_FP16 ? bp_kernel_info_fp16(n, weighted, code->crc_len <= 16)
                            : var               ? bp_kernel_info_fp32_var(n, var)
                                                : bp_kernel_info_fp32(n, weighted, code->crc_len <= 16);
+    if (next && !w && !var && precision == POLAR_FP32 && max_iters >= kBPCycleIters && B >= kBPCycleFrames) {
+        const BPKernelInfo c = bp_kernel_info_fp32_cyc(n, code->crc_len <= 16);
+        if (c.fn) k = c;
+    }
     if (!k.fn) return fail(POLAR_ERR_ARG, "no BP kernel for N = %d with these options", code->N);
     if (k.smem > 48 * 1024) {
         // above the default dynamic shared-memory limit (N = 4096); set once per kernel and device
