@@ -204,6 +204,7 @@ struct BPArgs {
     int row_bytes;
     int fixed_iters;           // run max_iters iterations regardless of the CRC
     int frame0;                // index of the launch's first frame (frames frame0 .. frame0 + B - 1)
+    int out16;                 // llr_u on a 16-byte boundary
 };
 
 // Message traits: FP32 (one frame per thread) or half2 (two frames per thread).
@@ -574,17 +575,26 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     static_assert(!SYNP || FPT == 2 || (PAIRS && R % 4 == 0), "packed syndromes: half2, or FP32 pairs");
     constexpr bool syn_packed = SYNP;
     constexpr bool syn_nodes = SYNP && FPT == 1;
+    // group 0's window is bits 0..b-1: a thread's nodes are R consecutive ones, inside one word of the
+    // frozen mask
+    static_assert(P::win(0) == 0 && 32 % R == 0 && R % 4 == 0, "consecutive nodes in group 0");
+    {
+        const int j0 = P::node(0, t, 0);
+        const uint32_t fz = C.frozen_bits[j0 >> 5] >> (j0 & 31);
 #pragma unroll
-    for (int k = 0; k < R; ++k) {
-        const int j = P::node(0, t, k);
-        const uint32_t col = C.colsyn[j];
-        if constexpr (syn_nodes) {
-            if (!(k & 1))
-                csyn[(k >> 2) * 2 * T + 2 * t + ((k >> 1) & 1)] = col | (C.colsyn[P::node(0, t, k + 1)] << 16);
-        } else {
-            csyn[k * T + t] = syn_packed ? (col | (col << 16)) : col;
+        for (int k = 0; k < R; k += 4) {
+            const uint4 col4 = *reinterpret_cast<const uint4*>(C.colsyn + j0 + k);
+            const uint32_t col[4] = {col4.x, col4.y, col4.z, col4.w};
+            if constexpr (syn_nodes) {
+                reinterpret_cast<uint2*>(csyn)[(k >> 2) * T + t] =
+                    make_uint2(col[0] | (col[1] << 16), col[2] | (col[3] << 16));
+            } else {
+#pragma unroll
+                for (int q = 0; q < 4; ++q) csyn[(k + q) * T + t] = syn_packed ? (col[q] | (col[q] << 16)) : col[q];
+            }
         }
-        Rc[1][k] = frozen_at(C.frozen_bits, j) ? Mv : MT::splat(0.0f);
+#pragma unroll
+        for (int k = 0; k < R; ++k) Rc[1][k] = (fz >> k) & 1u ? Mv : MT::splat(0.0f);
     }
     {
         const float* y0 = fr[0] >= 0 ? row(fr[0]) : nullptr;
@@ -659,11 +669,27 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
         uint32_t* pb = pbits + h * (N / 32);
         for (int i = t; i < N / 32; i += T) pb[i] = 0u;
         group_sync<T, SHARED_CTA>(slot);
+        {
+            // the payload positions among a thread's consecutive nodes are consecutive too: its bits are
+            // packed first and go into one word, or two
+            const short4* pp = reinterpret_cast<const short4*>(C.paypos + P::node(0, t, 0));
+            uint32_t v = 0;
+            int first = -1;
 #pragma unroll
-        for (int k = 0; k < R; ++k) {
-            const int j = P::node(0, t, k);
-            const int pos = C.paypos[j];
-            if (pos >= 0 && MT::neg(fadd(Lc[1][k], Rc[1][k]), h)) atomicOr(&pb[pos >> 5], 1u << (pos & 31));
+            for (int k = 0; k < R; k += 4) {
+                const short4 p4 = pp[k >> 2];
+                const int pos[4] = {p4.x, p4.y, p4.z, p4.w};
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    if (first < 0) first = pos[q];
+                    if (pos[q] >= 0 && MT::neg(fadd(Lc[1][k + q], Rc[1][k + q]), h)) v |= 1u << (pos[q] - first);
+                }
+            }
+            if (v) {
+                const uint64_t w = (uint64_t)v << (first & 31);
+                if ((uint32_t)w) atomicOr(&pb[first >> 5], (uint32_t)w);
+                if (w >> 32) atomicOr(&pb[(first >> 5) + 1], (uint32_t)(w >> 32));
+            }
         }
         group_sync<T, SHARED_CTA>(slot);
         // the packed payload has ceil(P/8) <= N/8 bytes; a wider output row (a mixed batch uses
@@ -681,9 +707,19 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
             }
         }
         if (a.llr_u) {
+            float* lu = a.llr_u + (size_t)frame * N + P::node(0, t, 0);
 #pragma unroll
-            for (int k = 0; k < R; ++k)
-                a.llr_u[(size_t)frame * N + P::node(0, t, k)] = MT::to_f(fadd(Lc[1][k], Rc[1][k]), h);
+            for (int k = 0; k < R; k += 4) {
+                float u[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) u[q] = MT::to_f(fadd(Lc[1][k + q], Rc[1][k + q]), h);
+                if (a.out16) {
+                    *reinterpret_cast<float4*>(lu + k) = make_float4(u[0], u[1], u[2], u[3]);
+                } else {
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) lu[k + q] = u[q];
+                }
+            }
         }
         if (a.llr_x) {
             // R[n+1] of the last R sweep, recomputed from R[n] and the channel column

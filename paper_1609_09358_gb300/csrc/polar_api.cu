@@ -409,6 +409,7 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
     const int groups = (B + fpt - 1) / fpt;
     const int F = k.groups_per_cta;
     int grid = (groups + F - 1) / F;
+    a.out16 = (reinterpret_cast<uintptr_t>(llr_u) & 15u) == 0;
     if (next) {
         // persistent: as many CTAs as are resident at once; groups refill from the counter
         int per_sm = 0;

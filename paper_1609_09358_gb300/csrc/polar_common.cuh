@@ -1,6 +1,7 @@
 // polar_common.cuh -- shared device-side definitions of the GB300 polar decoder.
 #pragma once
 
+#include <cstddef>
 #include <cstdint>
 #include <type_traits>
 #include <cuda_fp16.h>
@@ -15,9 +16,11 @@ constexpr int kMaxWords = kMaxN / 32;
 
 // Per-code tables derived on the host from (N, K, frozen, CRC) and kept in a static device
 // array, one slot per distinct code.
-struct DevCode {
+// The arrays start on 16-byte boundaries: the BP kernels read a thread's consecutive nodes in vectors.
+struct alignas(16) DevCode {
     int32_t N, n, K, P, c;
     uint32_t poly;
+    int32_t pad[2];
     uint32_t frozen_bits[kMaxWords];  // bit i of word i/32 set = node i frozen
     uint32_t decided_bits[kMaxWords]; // information positions CA-SCL decides without branching
     // Syndrome column of node i: x^(K-1-k) mod g(x) for the node's information index k, 0 for a
@@ -27,6 +30,8 @@ struct DevCode {
     int16_t paypos[kMaxN];    // payload position of node i, -1 for frozen and CRC nodes
     int16_t info_idx[kMaxN];  // node of information index k (k < K)
 };
+static_assert(offsetof(DevCode, colsyn) % 16 == 0 && offsetof(DevCode, paypos) % 16 == 0 && sizeof(DevCode) % 16 == 0,
+              "vector reads of the code tables");
 
 // ---------------------------------------------------------------------------- FP32 primitives
 // min-sum PE function g(a, b) = sign(a) sign(b) min(|a|, |b|) as one instruction: the magnitude
