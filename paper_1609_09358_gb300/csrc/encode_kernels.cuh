@@ -173,15 +173,30 @@ struct U4 {
     uint32_t x, y, z, w;
 };
 
-__device__ __forceinline__ U4 philox4x32_10(U4 c, uint32_t k0, uint32_t k1)
+// Round keys of a seed, made once on the host (kernel parameters: each round's key is an operand of its
+// XOR and costs no instruction).
+struct PhiloxKeys {
+    uint32_t k[10][2];
+};
+inline PhiloxKeys philox_keys(uint64_t seed)
+{
+    PhiloxKeys r;
+    uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
+    for (int i = 0; i < 10; ++i) {
+        r.k[i][0] = k0;
+        r.k[i][1] = k1;
+        k0 += 0x9E3779B9u;
+        k1 += 0xBB67AE85u;
+    }
+    return r;
+}
+
+__device__ __forceinline__ U4 philox4x32_10(U4 c, const PhiloxKeys& key)
 {
 #pragma unroll
     for (int r = 0; r < 10; ++r) {
-        const uint32_t lo0 = 0xD2511F53u * c.x, hi0 = __umulhi(0xD2511F53u, c.x);
-        const uint32_t lo1 = 0xCD9E8D57u * c.z, hi1 = __umulhi(0xCD9E8D57u, c.z);
-        c = U4{hi1 ^ c.y ^ k0, lo1, hi0 ^ c.w ^ k1, lo0};
-        k0 += 0x9E3779B9u;
-        k1 += 0xBB67AE85u;
+        const uint64_t p0 = (uint64_t)0xD2511F53u * c.x, p1 = (uint64_t)0xCD9E8D57u * c.z;
+        c = U4{(uint32_t)(p1 >> 32) ^ c.y ^ key.k[r][0], (uint32_t)p1, (uint32_t)(p0 >> 32) ^ c.w ^ key.k[r][1], (uint32_t)p0};
     }
     return c;
 }
@@ -189,12 +204,12 @@ __device__ __forceinline__ U4 philox4x32_10(U4 c, uint32_t k0, uint32_t k1)
 // Payload rows: a CTA fills the bytes of kPayRows rows in shared memory, one Philox block (128 bits) per
 // thread and step, and writes them out as one contiguous run in 16-byte stores.  (Rows are `bytes`
 // long and start at any residue; stores from the block's thread went out in bytes or half words, 18 us
-// per 10^5 rows of 62 bytes, now 9 us.)
+// per 10^5 rows of 62 bytes, now 7 us.)
 constexpr int kPayRows = 64;
 constexpr int kPayMaxBytes = 48 * 1024 / kPayRows;  // longer rows are written directly
-__device__ __forceinline__ U4 payload_block(uint64_t f, int blk, uint64_t seed)
+__device__ __forceinline__ U4 payload_block(uint64_t f, int blk, const PhiloxKeys& key)
 {
-    return philox4x32_10(U4{(uint32_t)blk, (uint32_t)f, 0u, (uint32_t)(f >> 32)}, (uint32_t)seed, (uint32_t)(seed >> 32));
+    return philox4x32_10(U4{(uint32_t)blk, (uint32_t)f, 0u, (uint32_t)(f >> 32)}, key);
 }
 // the block's bytes of a row of P bits (bytes = ceil(P / 8)); pad bits of the last byte are 0
 __device__ __forceinline__ void payload_store(uint8_t* row, int blk, int P, int bytes, const U4& r)
@@ -228,14 +243,14 @@ __device__ __forceinline__ void payload_store(uint8_t* row, int blk, int P, int 
     }
 }
 __global__ void __launch_bounds__(256)
-    random_payload_kernel(int B, int P, uint64_t seed, uint64_t frame0, uint8_t* __restrict__ out)
+    random_payload_kernel(int B, int P, const PhiloxKeys key, uint64_t frame0, uint8_t* __restrict__ out)
 {
     extern __shared__ __align__(16) uint8_t pay_smem[];
     const int nblocks = (P + 127) >> 7, bytes = (P + 7) >> 3;
     const int row0 = blockIdx.x * kPayRows, rows = min(kPayRows, B - row0);
     for (int i = threadIdx.x; i < rows * nblocks; i += blockDim.x) {
         const int b = i / nblocks, blk = i % nblocks;
-        payload_store(pay_smem + b * bytes, blk, P, bytes, payload_block(frame0 + (uint64_t)(row0 + b), blk, seed));
+        payload_store(pay_smem + b * bytes, blk, P, bytes, payload_block(frame0 + (uint64_t)(row0 + b), blk, key));
     }
     __syncthreads();
     uint8_t* dst = out + (size_t)row0 * bytes;
@@ -245,22 +260,22 @@ __global__ void __launch_bounds__(256)
     for (int i = 16 * vec + threadIdx.x; i < total; i += blockDim.x) dst[i] = pay_smem[i];
 }
 // Rows too long for shared memory: one thread per Philox block.
-__global__ void random_payload_direct_kernel(int B, int P, uint64_t seed, uint64_t frame0, uint8_t* __restrict__ out)
+__global__ void random_payload_direct_kernel(int B, int P, const PhiloxKeys key, uint64_t frame0, uint8_t* __restrict__ out)
 {
     const int nblocks = (int)(((long long)P + 127) >> 7), bytes = (int)(((long long)P + 7) >> 3);
     const long long gid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (long long)B * nblocks) return;
     const int b = (int)(gid / nblocks), blk = (int)(gid % nblocks);
-    payload_store(out + (size_t)b * bytes, blk, P, bytes, payload_block(frame0 + (uint64_t)b, blk, seed));
+    payload_store(out + (size_t)b * bytes, blk, P, bytes, payload_block(frame0 + (uint64_t)b, blk, key));
 }
 
 // One thread per Philox block (4 nodes) of one frame: Box-Muller on (w0, w1) and (w2, w3).  Bound by
 // instruction issue (ten Philox rounds, two logarithms, square roots and sine / cosine pairs per 16
 // bytes written).  N = 2^log2n, so frame and block come from shifts, and 2 / sigma^2 of a common sigma
 // (scale_all) from the host: with a 64-bit division and a float division per thread 10^5 frames of
-// N = 1024 took 260 us, now 232 us.
+// N = 1024 took 260 us, without 232, and with the round keys as kernel parameters 223.
 __global__ void awgn_llr_kernel(const uint8_t* __restrict__ codeword, int B, int log2n, float sigma_all, float scale_all,
-                                const float* __restrict__ sigmas, uint64_t seed, uint64_t frame0,
+                                const float* __restrict__ sigmas, const PhiloxKeys key, uint64_t frame0,
                                 float* __restrict__ llr)
 {
     const int N = 1 << log2n;
@@ -273,8 +288,7 @@ __global__ void awgn_llr_kernel(const uint8_t* __restrict__ codeword, int B, int
         scale = 2.0f / (sigma * sigma);
     }
     const uint64_t f = frame0 + (uint64_t)b;
-    const U4 r = philox4x32_10(U4{(uint32_t)blk, (uint32_t)f, 1u, (uint32_t)(f >> 32)}, (uint32_t)seed,
-                               (uint32_t)(seed >> 32));
+    const U4 r = philox4x32_10(U4{(uint32_t)blk, (uint32_t)f, 1u, (uint32_t)(f >> 32)}, key);
     const uint32_t e[2] = {r.x, r.z}, o[2] = {r.y, r.w};
     const uint8_t xb = codeword[(size_t)b * (N >> 3) + (blk >> 1)] >> ((blk & 1) * 4);
     float4 v;

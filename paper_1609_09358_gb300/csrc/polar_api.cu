@@ -592,9 +592,11 @@ int polar_random_payload(int32_t B, int32_t P, uint64_t seed, uint64_t frame0, u
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long bytes = ((long long)P + 7) / 8, total = B * (((long long)P + 127) / 128);
     if (bytes <= kPayMaxBytes)
-        random_payload_kernel<<<(B + kPayRows - 1) / kPayRows, 256, kPayRows * bytes, st>>>(B, P, seed, frame0, payload);
+        random_payload_kernel<<<(B + kPayRows - 1) / kPayRows, 256, kPayRows * bytes, st>>>(B, P, philox_keys(seed), frame0,
+                                                                                         payload);
     else
-        random_payload_direct_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, P, seed, frame0, payload);
+        random_payload_direct_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, P, philox_keys(seed), frame0,
+                                                                                       payload);
     POLAR_CUDA(cudaGetLastError());
     return POLAR_OK;
 }
@@ -608,7 +610,8 @@ int polar_awgn_llr(const uint8_t* codeword, int32_t B, int32_t N, float sigma, c
     if (!codeword || !llr) return fail(POLAR_ERR_ARG, "NULL codeword/llr");
     const long long total = (long long)B * (N / 4);
     awgn_llr_kernel<<<(unsigned)((total + 255) / 256), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        codeword, B, log2i(N), sigma, sigma_per_frame ? 0.0f : 2.0f / (sigma * sigma), sigma_per_frame, seed, frame0, llr);
+        codeword, B, log2i(N), sigma, sigma_per_frame ? 0.0f : 2.0f / (sigma * sigma), sigma_per_frame,
+        philox_keys(seed), frame0, llr);
     POLAR_CUDA(cudaGetLastError());
     return POLAR_OK;
 }
