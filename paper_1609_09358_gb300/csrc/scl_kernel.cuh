@@ -55,6 +55,7 @@ struct SCLArgs {
     float* scratch;    // per-warp slots of the global levels (null: all levels in shared memory)
     int row_bytes;
     int KS, KC;        // last LLR / partial-sum level kept in shared memory (single code)
+    int KSm, KCm;      // the same when a CTA decodes one frame at a time, with all its shared memory
     int warp_words;    // shared-memory words per warp
     int list_words;    // shared-memory words per list (two lists per warp when L <= 8)
     long long slot_words;  // global words per list
@@ -117,6 +118,23 @@ __host__ __device__ inline SCLPlan scl_plan(int N, int L, bool all_smem, int lis
     p.warp_words = lists * p.list_words + kSclWarpWords;
     p.slot_words = (long long)L * (N - (2 << p.KS)) + (long long)L * (scl_cssum(n + 1) - scl_cssum(p.KC + 1));
     return p;
+}
+// The levels in shared memory of a list that has `words` of it to itself (and fits there with the split
+// of scl_plan): as many LLR levels as leave room for the partial sums up to level 8, then the partial
+// sums.  With the per-warp split the partial sums of long codes and all but one or two LLR levels came
+// from L2, and a frame alone on its SM waits for every access (N = 4096, L = 32, 138 frames: 5.20 -> 5.15 ms with the exact-g BP).
+inline void scl_plan_cta(int N, int L, long long words, int* KS, int* KC)
+{
+    const int n = log2_host(N);
+    const auto fits = [&](int ks, int kc) {
+        return scl_smem_llr_words(ks, L) + L * kSclStage + scl_smem_c_words(kc, L) <= words;
+    };
+    int ks = 6, kc = 5;
+    while (ks + 1 <= n - 1 && fits(ks + 1, std::min(n, 8))) ++ks;
+    while (kc + 1 <= n && fits(ks, kc + 1)) ++kc;
+    if (ks < *KS || kc < *KC) return;
+    *KS = ks;
+    *KC = kc;
 }
 inline bool scl_fits_smem(int N, int L) { return 4LL * scl_plan(N, L, true).warp_words <= 80 * 1024; }
 constexpr int kSclWarpsPerSM = 32;
@@ -765,9 +783,24 @@ __device__ void scl_decode_frame(const SCLArgs& a, const DevCode& C, int frame, 
                     if (!whole) failed = r;
                 }
                 if (!whole) {
+                    int q = r;
+                    if ((f & 3u) == 3u) {
+                        // two or three frozen bits first: their metrics in one run
+                        leaf_f<2>(lf.l2, lf.l1);
+                        pm = __fsub_rn(pm, fminf(xmin(lf.l1[0], lf.l1[1]), 0.0f));
+                        pm = __fsub_rn(pm, fminf(__fadd_rn(lf.l1[1], lf.l1[0]), 0.0f));
+                        lf.c[0] = lf.c[1] = 0u;
+                        q = r + 2;
+                        if (f & 4u) {
+                            lf.l1[0] = __fadd_rn(lf.l2[2], lf.l2[0]);
+                            lf.l1[1] = __fadd_rn(lf.l2[3], lf.l2[1]);
+                            pm = __fsub_rn(pm, fminf(xmin(lf.l1[0], lf.l1[1]), 0.0f));
+                            q = r + 3;
+                        }
+                    }
                     // bit by bit
 #pragma unroll 1
-                    for (int q = r; q < r + 4; ++q) {
+                    for (; q < r + 4; ++q) {
                         float lam;
                         if (q & 1) {
                             lam = scl_g(lf.l1[0], lf.l1[1], lf.c[0], 0);
@@ -1016,8 +1049,8 @@ __device__ __forceinline__ void scl_warp_frame(const SCLArgs& a, int frame, int 
         S.KS = p.KS;
         S.KC = p.KC;
     } else {
-        S.KS = a.KS;
-        S.KC = a.KC;
+        S.KS = mw ? a.KSm : a.KS;
+        S.KC = mw ? a.KCm : a.KC;
     }
     // the LLR levels first: their 16-byte accesses need the list's 16-byte aligned start
     S.sA = reinterpret_cast<float*>(ws);
@@ -1039,7 +1072,7 @@ __device__ __forceinline__ void scl_run(const SCLArgs& a, int count, const bool 
     const int wid = mw ? 0 : threadIdx.x >> 5;
     uint32_t* wsw = smem + (size_t)wid * a.warp_words;
     uint32_t* ws = wsw + li * a.list_words;
-    uint32_t* scratch = wsw + a.warp_words - kSclWarpWords;
+    uint32_t* scratch = wsw + (mw ? (blockDim.x >> 5) : 1) * a.warp_words - kSclWarpWords;
     uint8_t* selc = reinterpret_cast<uint8_t*>(scratch);
     uint32_t* ptab = scratch + kSclScratch;
     float* slot = a.scratch
@@ -1123,6 +1156,9 @@ cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int list_words_
     const size_t wb = (size_t)a.warp_words * 4;
     while (W > 1 && (size_t)W * wb > 200 * 1024) W >>= 1;
     const size_t smem = (size_t)W * wb;
+    a.KSm = a.KS;
+    a.KCm = a.KC;
+    if (!all_smem) scl_plan_cta(N, L, (long long)W * a.warp_words - kSclWarpWords, &a.KSm, &a.KCm);
     const bool two = L > 16;
     const void* fn = lists == 2 ? (const void*)scl_kernel<false, 16>
                                 : (two ? (const void*)scl_kernel<true, 32> : (const void*)scl_kernel<false, 32>);
