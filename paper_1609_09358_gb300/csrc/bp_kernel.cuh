@@ -52,15 +52,22 @@ struct BPPlan {
     // in every group the 5 lane bits of the thread index land on node bits whose addresses are
     // 1, 2, 4, 8, 16 modulo 32 in some order -- for group 1 that takes node bits 0, 1, 2, 8, 9
     // with b = 3, and 0, 1, 2, 3, 9 with b = 4 (a search over the plans finds such bits for
-    // N >= 1024 with b = 3 and b = 4 only).  The other plans
-    // keep an XOR swizzle of index bits 5..7 into the bank bits (one XOR per access).
-    static constexpr bool PAD = (LOGR == 3 && LOGN >= 10) || (LOGR == 4 && LOGN >= 10);
+    // N >= 1024 with b = 3 and b = 4 only).  N = 256 and 512 with b = 3 (SMALL) take additive addresses
+    // too, j plus 1, 10, 20, 32 for index bits 5..8, which leave group 1's accesses two to a bank: no
+    // additive layout is conflict-free there, and an XOR per access, free of conflicts, was worse -- it
+    // runs on the comparison pipe, the kernels' limit (86% busy at N = 512 against 37% of the
+    // shared-memory pipe; BP with LLR outputs, 20 011 frames, 5 iterations: 146 -> 123 us).  The plans with
+    // b = 2 keep an XOR swizzle of index bits 5 and 6 into the bank bits.
+    static constexpr bool PAD = (LOGR == 3 && LOGN >= 8) || (LOGR == 4 && LOGN >= 10);
+    static constexpr bool SMALL = LOGR == 3 && LOGN < 10;
+    // lanes of a warp that may share a bank in group g
+    __host__ __device__ static constexpr int ways(int g) { return SMALL && g == 1 ? 2 : 1; }
     // node bit receiving thread-index bit q in group g: the non-window bits in ascending order,
     // except that group 1 of a PAD plan puts lane bits 3, 4 on node bits 8, 9 (b = 3) or lane
     // bit 4 on node bit 9 (b = 4)
     __host__ __device__ static constexpr int tbit(int g, int q)
     {
-        if (PAD && LOGR == 3 && g == 1)  // window 3..5: thread bits -> node bits 0 1 2 8 9 6 7 10 ...
+        if (PAD && !SMALL && LOGR == 3 && g == 1)  // window 3..5: thread bits -> node bits 0 1 2 8 9 6 7 10 ...
             return q < 3 ? q : q < 5 ? q + 5 : q < 7 ? q + 1 : q + 3;
         if (PAD && LOGR == 4 && g == 1)  // window 4..7: thread bits -> node bits 0 1 2 3 9 8 10 11
             return q < 4 ? q : q == 4 ? 9 : q == 5 ? 8 : q + 4;
@@ -92,17 +99,16 @@ struct BPPlan {
         for (int i = LOGN; i > s; --i) c += lcross(i);
         return c;
     }
-    // XOR swizzle of the non-PAD plans: index bits 5..7 into the bank bits
-    __host__ __device__ static constexpr int swz(int j)
+    // XOR swizzle of the non-PAD plans: index bits 5 and 6 into the bank bits
+    __host__ __device__ static constexpr int swz(int j) { return j ^ (((j >> 5) & 1) * 5) ^ (((j >> 6) & 1) * 26); }
+    __host__ __device__ static constexpr int addr(int j)
     {
-        if constexpr (LOGR == 3)
-            return j ^ (((j >> 5) & 1) * 1) ^ (((j >> 6) & 1) * 10) ^ (((j >> 7) & 1) * 20);
-        else
-            return j ^ (((j >> 5) & 1) * 5) ^ (((j >> 6) & 1) * 26);
+        return !PAD ? swz(j)
+            : SMALL ? j + ((j >> 5) & 1) + ((j >> 6) & 1) * 10 + ((j >> 7) & 1) * 20 + ((j >> 8) & 1) * 32
+                    : j + (j >> 5) + (j >> 10);
     }
-    __host__ __device__ static constexpr int addr(int j) { return PAD ? j + (j >> 5) + (j >> 10) : swz(j); }
     // words of one exchange buffer
-    static constexpr int XW = PAD ? ((N + (N >> 5) + (N >> 10)) + 3) & ~3 : N;
+    static constexpr int XW = !PAD ? N : SMALL ? N + (LOGN - 7) * 32 : ((N + (N >> 5) + (N >> 10)) + 3) & ~3;
 };
 
 // Compile-time checks of a plan, one group at a time (each its own constant expression, so the
@@ -123,18 +129,16 @@ constexpr bool plan_group_bijective()
 template <class P, int G, int K>
 constexpr bool plan_group_banks()
 {
-    // register K of the 32 threads of every warp: distinct banks; PAD plans: the address splits
-    // into the thread's base and the register's offset
+    // register K of the 32 threads of every warp: distinct banks (at most ways(G) threads to a bank);
+    // PAD plans: the address splits into the thread's base and the register's offset
     for (int w = 0; w < P::NW; ++w) {
-        uint32_t banks = 0;
+        int banks[32] = {};
         for (int l = 0; l < 32 && w * 32 + l < P::T; ++l) {
             const int t = w * 32 + l;
             const int a = P::addr(P::node(G, t, K));
             if (a < 0 || a >= P::XW) return false;
             if (P::PAD && a != P::addr(P::tpart(G, t)) + P::addr(P::kpart(G, K))) return false;
-            const uint32_t bit = 1u << (a & 31);
-            if (banks & bit) return false;
-            banks |= bit;
+            if (++banks[a & 31] > P::ways(G)) return false;
         }
     }
     return true;
