@@ -187,6 +187,11 @@ __device__ __forceinline__ MSG xget(const MSG* xb, const int* xbase, int t, int 
         return xb[P::swz(P::node(G, t, k))];
 }
 
+// CYC: below this balance (iterations skipped less a sixteenth of those run, summed over the frames) the
+// kernel takes no more frames and leaves the rest to the plain one: about the first frames of the
+// groups that start together, if they run long and do not repeat.
+constexpr int kBPBalance = -4096;
+
 struct BPArgs {
     const float* llr;
     int B;
@@ -209,6 +214,7 @@ struct BPArgs {
     int fixed_iters;           // run max_iters iterations regardless of the CRC
     int frame0;                // index of the launch's first frame (frames frame0 .. frame0 + B - 1)
     int out16;                 // llr_u on a 16-byte boundary
+    int* balance;              // CYC: iterations skipped less a sixteenth of those run, over the launch
 };
 
 // Message traits: FP32 (one frame per thread) or half2 (two frames per thread).
@@ -532,10 +538,14 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     // not pass max_iters.  Everything written out is what the skipped iterations would have given.
     // This happens where the stop decision already parts the iteration (DEFER): the messages that
     // matter there are the columns R[2..SC+1] of the sweep under way (the last one in the exchange
-    // buffer) and L[SC+2..n].  At the loop's start, where they would be L[2..n], the extra branch kept
-    // the compiler from overlapping the syndrome with the next sweep and cost 10% of every iteration;
-    // here the kernel's iterations are 7% longer than the plain one's (launch_bp chooses).
-    // Measured: the production hybrid (N = 1024, K = 512, 10^5 frames, 2.5 dB) 4.33 -> 3.91 ms.
+    // buffer) and L[SC+2..n].  The kernel's iterations are 7% longer than the plain one's, most of it
+    // register copies that the rare blocks' needs bring into the loop (5% more instructions; 10% longer
+    // with the look at the loop's start, where the state would be L[2..n]).  That pays where failing frames
+    // repeat (2 dB and up) and not where they wander (11% repeat at 1.5 dB, fewer below), so a launch
+    // keeps the balance of what it skips and ends early if it falls; launch_bp follows it with the
+    // plain kernel on the same counter.  BP and a list of one, 10^5 frames, i_max = 200, plain / both:
+    // 40.35 / 40.54 ms at 1.0 dB, 29.1 / 29.3 at 1.5, 11.7 / 11.2 at 2.0, 4.07 / 3.69 at 2.5,
+    // 2.27 / 2.14 at 3.0, 1.64 / 1.66 at 3.5.
     constexpr bool CYC = (VAR & 4) != 0;
     static_assert(!CYC || (VAR == 4 && T > 32 && std::is_same<Src, CounterSource>::value), "repeats: plain FP32 min-sum");
     uint32_t* pbits = synp + 4 * NW;                       // [2 frame][N/32]
@@ -552,12 +562,19 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     int cue = 0;  // equal syndromes in a row (negative: looks to wait after a miss)
     bool is_saved = false;
     uint32_t last_syn = 0;
+    int skipped = 0;  // iterations of this frame
 
     // Frames of this group: half h (h < FPT) decodes frame fr[h]; when it stops it fetches the
     // next frame from the source.
     auto fetch = [&]() -> int { return src.template fetch<T, SHARED_CTA>(slot, t, fetched); };
     auto row = [&](int f) -> const float* { return a.llr + (a.llr_off ? a.llr_off[f] : (long long)f * N); };
     int fr[2] = {-1, -1}, itc[2] = {0, 0};
+    if constexpr (CYC) {
+        // the balance may have fallen in an earlier launch on the same frames' counters
+        if (t == 0) fetched[1] = *static_cast<volatile int*>(a.balance);
+        group_sync<T, SHARED_CTA>(slot);
+        if (fetched[1] < kBPBalance) return;
+    }
     fr[0] = fetch();
     if constexpr (FPT == 2) fr[1] = fetch();
     if (fr[0] < 0 && fr[1] < 0) return;  // uniform over the group
@@ -1001,7 +1018,8 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                                 cue = -4;
                                 if (__syncthreads_and(diff == 0u)) {
                                     // this iteration and the three before it, none of which stopped, repeat
-                                    itc[0] += (a.max_iters - itc[0]) & ~3;
+                                    skipped = (a.max_iters - itc[0]) & ~3;
+                                    itc[0] += skipped;
                                     stop = itc[0] >= a.max_iters;
                                 }
                             } else {
@@ -1015,9 +1033,19 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                     }
                     if (stop) {
                         finalize(0, itc[0], ok);
+                        if constexpr (CYC) {
+                            if (t == 0) {
+                                const int gain = min(skipped, 1024) - ((itc[0] - skipped) >> 4);
+                                const int now = atomicAdd(a.balance, gain);
+                                if (now > (1 << 24)) atomicAdd(a.balance, -gain);  // far from the limit
+                                fetched[1] = now;
+                            }
+                            group_sync<T, SHARED_CTA>(slot);
+                            if (fetched[1] < kBPBalance) break;
+                            cue = skipped = 0;
+                            is_saved = false;
+                        }
                         refill(0);
-                        cue = 0;
-                        is_saved = false;
                         if (fr[0] < 0) break;
                         continue;  // the new frame starts its first R sweep
                     }

@@ -186,7 +186,7 @@ struct ChunkHdr {
     int fail_count;
     int scl_next;
     int bp_next;
-    int pad;
+    int bp_balance;  // BPArgs::balance
 };
 static size_t hybrid_chunk_header_bytes(int) { return 256; }
 
@@ -343,18 +343,48 @@ static int bp_variant(int precision)
 static int bp_message(int precision) { return precision & ~(POLAR_G_EXACT | POLAR_STOP_REENCODE | POLAR_WMS_UNIT); }
 
 // From these iteration limits and batch sizes on the FP32 min-sum kernel that recognises repeating frames
-// is taken (N = 1024): its iterations take 7% longer, and it needs about 25 to find a repetition, so it
-// pays only if failing frames would run on well beyond that and if other frames wait for their place (a
-// batch that is resident at once ends with its longest frame, and not every failing frame repeats).
-constexpr int kBPCycleIters = 48, kBPCycleFrames = 2048;
+// goes first (N = 1024).  It needs about 25 iterations to find a repetition, so failing frames have to
+// run on well beyond that (at 50 every batch measured 2 to 6% slower); and where it gives up (see CYC in
+// bp_kernel.cuh) its last frames overlap nothing for up to max_iters iterations, 0.16 ms at 200, which
+// has to be little of the whole batch (37 frames, all resident at once: 352 -> 368 us with it).
+constexpr int kBPCycleIters = 150, kBPCycleFrames = 16384;
+
+static int launch_bp_kernel(const BPKernelInfo& k, BPArgs& a, int fpt, cudaStream_t stream)
+{
+    if (k.smem > 48 * 1024) {
+        // above the default dynamic shared-memory limit; set once per kernel and device
+        static std::mutex m;
+        static std::vector<std::pair<int, const void*>> done;
+        int dev = 0;
+        POLAR_CUDA(cudaGetDevice(&dev));
+        std::lock_guard<std::mutex> lock(m);
+        if (std::find(done.begin(), done.end(), std::make_pair(dev, k.fn)) == done.end()) {
+            POLAR_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
+            done.push_back(std::make_pair(dev, k.fn));
+        }
+    }
+    const int groups = (a.B + fpt - 1) / fpt, F = k.groups_per_cta;
+    int grid = (groups + F - 1) / F;
+    if (a.next) {
+        // persistent: as many CTAs as are resident at once; groups refill from the counter
+        int per_sm = 0;
+        const cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem);
+        if (e != cudaSuccess) return cuda_fail(e, "bp occupancy");
+        grid = std::min(grid, std::max(1, per_sm) * scl_sm_count());
+    }
+    void* args[] = {&a};
+    const cudaError_t e = cudaLaunchKernel(k.fn, dim3(grid), dim3(k.threads), args, k.smem, stream);
+    return e == cudaSuccess ? POLAR_OK : cuda_fail(e, "bp_kernel launch");
+}
 
 static int launch_bp(const DevCode* dcode, const polar_code* code, const float* llr, int B, int max_iters,
                      float llr_max, int precision, const void* w, int w_iters, uint8_t* bits, uint8_t* status,
                      uint16_t* iters, float* llr_u, float* llr_x, int* fail_count, int* fail_list,
                      cudaStream_t stream, int* fail_total = nullptr, int* next = nullptr, int fixed_iters = 0,
-                     int frame0 = 0)
+                     int frame0 = 0, int* balance = nullptr, int batch = 0)
 {
     BPArgs a{};
+    a.balance = balance;
     a.frame0 = frame0;
     a.fixed_iters = fixed_iters;
     a.fail_total = fail_total;
@@ -385,42 +415,19 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
     // learned scales: the half2 form with both frames of a register on the same iteration when
     // the caller vouches for scales within [-1, 1] and every iteration is a learned one
     const int weighted = !w ? 0 : (unit && precision == POLAR_FP16 && max_iters <= w_iters) ? 2 : 1;
-    BPKernelInfo k = precision == POLAR_FP16 ? bp_kernel_info_fp16(n, weighted, code->crc_len <= 16)
+    const BPKernelInfo k = precision == POLAR_FP16 ? bp_kernel_info_fp16(n, weighted, code->crc_len <= 16)
                            : var               ? bp_kernel_info_fp32_var(n, var)
                                                : bp_kernel_info_fp32(n, weighted, code->crc_len <= 16);
-    if (next && !w && !var && precision == POLAR_FP32 && max_iters >= kBPCycleIters && B >= kBPCycleFrames) {
-        const BPKernelInfo c = bp_kernel_info_fp32_cyc(n, code->crc_len <= 16);
-        if (c.fn) k = c;
-    }
     if (!k.fn) return fail(POLAR_ERR_ARG, "no BP kernel for N = %d with these options", code->N);
-    if (k.smem > 48 * 1024) {
-        // above the default dynamic shared-memory limit (N = 4096); set once per kernel and device
-        static std::mutex m;
-        static std::vector<std::pair<int, const void*>> done;
-        int dev = 0;
-        POLAR_CUDA(cudaGetDevice(&dev));
-        std::lock_guard<std::mutex> lock(m);
-        if (std::find(done.begin(), done.end(), std::make_pair(dev, k.fn)) == done.end()) {
-            POLAR_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
-            done.push_back(std::make_pair(dev, k.fn));
-        }
-    }
-    const int fpt = precision == POLAR_FP16 ? 2 : 1;
-    const int groups = (B + fpt - 1) / fpt;
-    const int F = k.groups_per_cta;
-    int grid = (groups + F - 1) / F;
     a.out16 = (reinterpret_cast<uintptr_t>(llr_u) & 15u) == 0;
-    if (next) {
-        // persistent: as many CTAs as are resident at once; groups refill from the counter
-        int per_sm = 0;
-        cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem);
-        if (e != cudaSuccess) return cuda_fail(e, "bp occupancy");
-        grid = std::min(grid, std::max(1, per_sm) * scl_sm_count());
-    }
+    const int fpt = precision == POLAR_FP16 ? 2 : 1;
     ProfScope prof(0, stream);
-    void* args[] = {&a};
-    const cudaError_t e = cudaLaunchKernel(k.fn, dim3(grid), dim3(k.threads), args, k.smem, stream);
-    return e == cudaSuccess ? POLAR_OK : cuda_fail(e, "bp_kernel launch");
+    const bool cyc = next && balance && !w && !var && precision == POLAR_FP32 && max_iters >= kBPCycleIters &&
+                     batch >= kBPCycleFrames;
+    const BPKernelInfo first = cyc ? bp_kernel_info_fp32_cyc(n, code->crc_len <= 16) : BPKernelInfo{nullptr, 0, 0, 0};
+    int rc = POLAR_OK;
+    if (first.fn) rc = launch_bp_kernel(first, a, fpt, stream);
+    return rc ? rc : launch_bp_kernel(k, a, fpt, stream);
 }
 
 static int check_bp_args(const polar_code* code, const float* llr, int B, int max_iters, float llr_max,
@@ -683,7 +690,7 @@ int hybrid_decode(const polar_code* code, const float* llr, int32_t B, int32_t m
     void* scratch = reinterpret_cast<char*>(list) + align_up(sizeof(int) * (size_t)B, 256);
     POLAR_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes + sizeof(ChunkHdr), st));
     if ((rc = launch_bp(d, code, llr, B, max_iters, llr_max, precision, wms_scales, wms_iters, bits, status, iters,
-                        nullptr, nullptr, &hdr->fail_count, list, st, total, &hdr->bp_next)))
+                        nullptr, nullptr, &hdr->fail_count, list, st, total, &hdr->bp_next, 0, 0, &hdr->bp_balance, B)))
         return rc;
     return launch_scl(d, code, llr, B, L, bits, status, list, &hdr->fail_count, &hdr->scl_next, scratch, st);
 }
@@ -746,7 +753,8 @@ int hybrid_decode_host(const polar_code* code, const float* llr_host, int32_t B,
         POLAR_CUDA(cudaEventRecord(evc, stc));
         POLAR_CUDA(cudaStreamWaitEvent(st, evc, 0));
         rc = launch_bp(d, code, llr_d, nb, max_iters, llr_max, precision, wms_scales, wms_iters, bits_d, status_d,
-                       iters_d, nullptr, nullptr, &hdr->fail_count, list, st, total, counters + c, 0, b0);
+                       iters_d, nullptr, nullptr, &hdr->fail_count, list, st, total, counters + c, 0, b0,
+                       &hdr->bp_balance, B);
     }
     if (rc == POLAR_OK && (rc = event(&ev1)) == POLAR_OK) {
         POLAR_CUDA(cudaEventRecord(ev1, st1));
