@@ -146,7 +146,7 @@ static int code_slot(const polar_code* code, cudaStream_t stream, const DevCode*
         dc.init = true;
     }
     for (size_t s = 0; s < dc.host.size(); ++s) {
-        if (memcmp(&dc.host[s], &d, sizeof d) == 0) {
+        if (memcmp(&dc.host[s], &d, offsetof(DevCode, xsyn)) == 0) {
             *out = dc.base + s;
             return POLAR_OK;
         }
@@ -155,6 +155,12 @@ static int code_slot(const polar_code* code, cudaStream_t stream, const DevCode*
         return fail(POLAR_ERR_CAPACITY, "more than %d distinct codes used on device %d", POLAR_MAX_CODES, dev);
     dc.host.push_back(d);
     const size_t s = dc.host.size() - 1;
+    // u_j is the XOR of the x_i whose index i contains j's bits, so x_i's column is that of every j in i
+    uint32_t* xs = dc.host[s].xsyn;
+    std::copy(d.colsyn, d.colsyn + kMaxN, xs);
+    for (int D = 1; D < d.N; D <<= 1)
+        for (int i = 0; i < d.N; ++i)
+            if (i & D) xs[i] ^= xs[i ^ D];
     cudaError_t e = cudaMemcpyAsync(dc.base + s, &dc.host[s], sizeof(DevCode), cudaMemcpyHostToDevice, stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
     if (e != cudaSuccess) {

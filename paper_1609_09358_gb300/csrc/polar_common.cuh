@@ -29,8 +29,12 @@ struct alignas(16) DevCode {
     uint32_t colsyn[kMaxN];
     int16_t paypos[kMaxN];    // payload position of node i, -1 for frozen and CRC nodes
     int16_t info_idx[kMaxN];  // node of information index k (k < K)
+    // The same for the bits of the codeword x: with u = x G the remainder is the XOR of xsyn over the
+    // bits of x that are 1.  Follows from the fields above: made once per slot, left out of their
+    // comparison.
+    uint32_t xsyn[kMaxN];
 };
-static_assert(offsetof(DevCode, colsyn) % 16 == 0 && offsetof(DevCode, paypos) % 16 == 0 && sizeof(DevCode) % 16 == 0,
+static_assert(offsetof(DevCode, xsyn) % 16 == 0 && offsetof(DevCode, colsyn) % 16 == 0 && offsetof(DevCode, paypos) % 16 == 0 && sizeof(DevCode) % 16 == 0,
               "vector reads of the code tables");
 
 // ---------------------------------------------------------------------------- FP32 primitives

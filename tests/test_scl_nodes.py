@@ -71,3 +71,23 @@ def test_whole_nodes_bit_exact(which, ties, L):
         assert np.array_equal(status.cpu().numpy(), np.tile(ref["status"], times))
         assert np.array_equal(api.unpack_bits(bits.cpu().numpy(), code.P),
                               np.tile(oracle.payload_of(ref["u_hat"], ocode), (times, 1)))
+
+
+@pytest.mark.parametrize("L", [2, 8, 32])
+@pytest.mark.parametrize("N,K,c", [(128, 64, 8), (1024, 512, 16), (4096, 2048, 16)])
+def test_crc_selection_over_all_paths(N, K, c, L):
+    """Frames at a signal where most fail: every path's CRC is tested before the best one is output,
+    and with 8 CRC bits some frames end on a path that is not the best."""
+    ocode = fr.oracle_code(N, K, c)
+    B = 64 if N == 128 else 6
+    _, llr = fr.frames(ocode, -1.0, B, seed=900 + L)
+    ref = oracle.scl_decode(llr, ocode, L, "f32")
+    assert (ref["status"] != ref["status"].min()).any() or N > 128
+    code = api.PolarCode(N, K, c, ocode.frozen.copy(), ocode.crc_poly)
+    ws = torch.empty(api.polar_workspace_bytes(code, B, L, api.POLAR_OP_SCL), dtype=torch.uint8, device="cuda")
+    bits = torch.zeros((B, code.row_bytes), dtype=torch.uint8, device="cuda")
+    status = torch.zeros(B, dtype=torch.uint8, device="cuda")
+    api.scl_decode(code, torch.from_numpy(llr).cuda(), L, bits, status, ws)
+    torch.cuda.synchronize()
+    assert np.array_equal(status.cpu().numpy(), ref["status"])
+    assert np.array_equal(api.unpack_bits(bits.cpu().numpy(), code.P), oracle.payload_of(ref["u_hat"], ocode))
