@@ -368,6 +368,8 @@ def main():
     ops10 = 10 * n * N + K
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12, "unit": "Top/s",
                 "frac": achieved / peak_ops, "traffic": traffic, "kernel": "bp_kernel",
+                "iterations": "as reported; whole periods of repeating frames are skipped, so achieved "
+                              "counts operations that were not run",
                 "ops_per_frame_iter": ops_per_frame_iter, "bp_avg_ms": bp_avg_ms,
                 "peak_basis": "%d SMs x %d lanes x %.0f MHz (sm_max_mhz of MEASURED_PEAKS.json); 6 ops per PE "
                               "half-iteration = 3 comparison-pipe instructions at half rate" % (sms, lanes, sm_max_mhz),
