@@ -93,10 +93,11 @@ __global__ void __launch_bounds__(kEncWarps * 32)
     __syncthreads();
     // widest access every payload row allows: its start and length in bytes decide
     const int align = (int)((reinterpret_cast<uintptr_t>(payload) | (uintptr_t)pay_bytes) & 3u);
-    const int stride = gridDim.x * kEncWarps * frames;
-    for (int f0 = (blockIdx.x * kEncWarps + (threadIdx.x >> 5)) * frames; f0 < B; f0 += stride) {
-        const int frame = f0 + slot;
-        const bool live = frame < B;
+    // (unsigned: the last step of a grid may pass 2^31)
+    const uint32_t frames_all = (uint32_t)B, stride = gridDim.x * kEncWarps * frames;
+    for (uint32_t f0 = (blockIdx.x * kEncWarps + (threadIdx.x >> 5)) * frames; f0 < frames_all; f0 += stride) {
+        const uint32_t frame = f0 + slot;
+        const bool live = frame < frames_all;
         const uint8_t* pay = payload + (size_t)(live ? frame : f0) * pay_bytes;
         uint32_t crc = 0u;
 #pragma unroll

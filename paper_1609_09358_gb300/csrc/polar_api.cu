@@ -585,7 +585,7 @@ int polar_encode(const polar_code* code, const uint8_t* payload, int32_t B, uint
     if (!codeword || (!payload && code->K > code->crc_len)) return fail(POLAR_ERR_ARG, "NULL payload/codeword");
     // enough CTAs for several per SM; each loops over the batch and prepares the code's tables once
     const int N = code->N, P = code->K - code->crc_len, per_cta = kEncWarps * (N >= 1024 ? 1 : 1024 / N);
-    const int grid = std::min((B + per_cta - 1) / per_cta, 4 * scl_sm_count());
+    const int grid = (int)std::min(((long long)B + per_cta - 1) / per_cta, 4LL * scl_sm_count());
     const size_t smem = enc_smem_bytes(N, P);
     const void* fn = N <= 1024   ? (const void*)encode_kernel<1>
                      : N == 2048 ? (const void*)encode_kernel<2>

@@ -1,0 +1,39 @@
+"""Frame generation at the largest batch an int32 count allows: frame indices next to 2^31."""
+import numpy as np
+import pytest
+
+import oracle
+from tests import frames as fr
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+from paper_1609_09358_gb300 import api, build  # noqa: E402
+
+BATCH = 2**31 - 1
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    api.load()
+    if torch.cuda.mem_get_info()[0] < 64 << 30:
+        pytest.skip("needs 64 GB of device memory")
+    yield
+    torch.cuda.empty_cache()
+
+
+def test_encoder_at_the_largest_batch():
+    """One byte of payload and 16 of codeword per frame; every row against the codeword of its byte."""
+    ocode = fr.oracle_code(128, 16, 8, design_rate=8 / 128)
+    pay = torch.arange(256, dtype=torch.uint8, device="cuda").repeat(2**23)[:BATCH].view(BATCH, 1)
+    cw = torch.zeros((BATCH, 16), dtype=torch.uint8, device="cuda")
+    api.polar_encode(fr.api_code(ocode), pay, cw)
+    bits = api.unpack_bits(np.arange(256, dtype=np.uint8).reshape(256, 1), 8)
+    row = torch.from_numpy(api.pack_bits(oracle.encode_batch(bits, ocode))).cuda()
+    for b in range(0, BATCH, 2**28):  # a multiple of 256 rows
+        part = cw[b:b + 2**28]
+        whole = part.shape[0] // 256 * 256
+        assert bool((part[:whole].view(-1, 256, 16) == row).all())
+        assert torch.equal(part[whole:], row[:part.shape[0] - whole])
