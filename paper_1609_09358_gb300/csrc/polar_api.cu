@@ -605,8 +605,8 @@ int polar_random_payload(int32_t B, int32_t P, uint64_t seed, uint64_t frame0, u
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const long long bytes = ((long long)P + 7) / 8, total = B * (((long long)P + 127) / 128);
     if (bytes <= kPayMaxBytes)
-        random_payload_kernel<<<(B + kPayRows - 1) / kPayRows, 256, kPayRows * bytes, st>>>(B, P, philox_keys(seed), frame0,
-                                                                                         payload);
+        random_payload_kernel<<<(unsigned)(((long long)B + kPayRows - 1) / kPayRows), 256, kPayRows * bytes, st>>>(
+            B, P, philox_keys(seed), frame0, payload);
     else
         random_payload_direct_kernel<<<(unsigned)((total + 255) / 256), 256, 0, st>>>(B, P, philox_keys(seed), frame0,
                                                                                        payload);

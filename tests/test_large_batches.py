@@ -3,6 +3,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_1609_09358_gb300 import inputs
 from tests import frames as fr
 
 torch = pytest.importorskip("torch")
@@ -37,3 +38,11 @@ def test_encoder_at_the_largest_batch():
         whole = part.shape[0] // 256 * 256
         assert bool((part[:whole].view(-1, 256, 16) == row).all())
         assert torch.equal(part[whole:], row[:part.shape[0] - whole])
+
+
+def test_payload_at_the_largest_batch():
+    out = torch.full((BATCH, 1), 0xFF, dtype=torch.uint8, device="cuda")
+    api.polar_random_payload(BATCH, 7, 77, 5, out)
+    for b in (0, 2**31 - 200):  # the second range ends with the last, partial block of rows
+        n = min(199, BATCH - b)
+        assert np.array_equal(out[b:b + n].cpu().numpy(), api.pack_bits(inputs.payload_bits(77, 5 + b, n, 7)))
