@@ -357,18 +357,7 @@ constexpr int kBPCycleIters = 150, kBPCycleFrames = 16384;
 
 static int launch_bp_kernel(const BPKernelInfo& k, BPArgs& a, int fpt, cudaStream_t stream)
 {
-    if (k.smem > 48 * 1024) {
-        // above the default dynamic shared-memory limit; set once per kernel and device
-        static std::mutex m;
-        static std::vector<std::pair<int, const void*>> done;
-        int dev = 0;
-        POLAR_CUDA(cudaGetDevice(&dev));
-        std::lock_guard<std::mutex> lock(m);
-        if (std::find(done.begin(), done.end(), std::make_pair(dev, k.fn)) == done.end()) {
-            POLAR_CUDA(cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem));
-            done.push_back(std::make_pair(dev, k.fn));
-        }
-    }
+    POLAR_CUDA(raise_smem_limit(k.fn, k.smem));
     const int groups = (a.B + fpt - 1) / fpt, F = k.groups_per_cta;
     int grid = (groups + F - 1) / F;
     if (a.next) {
@@ -590,7 +579,7 @@ int polar_encode(const polar_code* code, const uint8_t* payload, int32_t B, uint
     const void* fn = N <= 1024   ? (const void*)encode_kernel<1>
                      : N == 2048 ? (const void*)encode_kernel<2>
                                  : (const void*)encode_kernel<4>;
-    if (smem > 48 * 1024) POLAR_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    POLAR_CUDA(raise_smem_limit(fn, smem));
     int pay_bytes = (P + 7) / 8;
     void* args[] = {&d, &payload, &B, &pay_bytes, &codeword};
     POLAR_CUDA(cudaLaunchKernel(fn, dim3(grid), dim3(kEncWarps * 32), args, smem, st));
@@ -1112,7 +1101,7 @@ int mix_bp(const polar_code* codes, int ncodes, const DevCode* const* dcodes, co
         packed = packed && codes[c].crc_len <= 16;
     }
     const void* fn = bp_mixed_fn(precision, packed);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(fn, smem);
     if (e != cudaSuccess) return cuda_fail(e, "bp_mixed_kernel attribute");
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, kMixBlock, smem);

@@ -3,7 +3,10 @@
 
 #include <cstddef>
 #include <cstdint>
+#include <map>
+#include <mutex>
 #include <type_traits>
+#include <utility>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
@@ -36,6 +39,25 @@ struct alignas(16) DevCode {
 };
 static_assert(offsetof(DevCode, xsyn) % 16 == 0 && offsetof(DevCode, colsyn) % 16 == 0 && offsetof(DevCode, paypos) % 16 == 0 && sizeof(DevCode) % 16 == 0,
               "vector reads of the code tables");
+
+// Lets kernel `fn` take `bytes` of dynamic shared memory on the current device.  The limit is one value
+// per kernel and device, shared by all host threads and by launches of different sizes, so it only
+// grows: lowering it could fail a launch that another thread has just raised it for.
+inline cudaError_t raise_smem_limit(const void* fn, size_t bytes)
+{
+    if (bytes <= 48 * 1024) return cudaSuccess;  // the default limit
+    static std::mutex m;
+    static std::map<std::pair<int, const void*>, size_t> limits;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(m);
+    size_t& limit = limits[std::make_pair(dev, fn)];
+    if (bytes <= limit) return cudaSuccess;
+    e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    if (e == cudaSuccess) limit = bytes;
+    return e;
+}
 
 // ---------------------------------------------------------------------------- FP32 primitives
 // min-sum PE function g(a, b) = sign(a) sign(b) min(|a|, |b|) as one instruction: the magnitude

@@ -1155,7 +1155,7 @@ cudaError_t scl_launch(SCLArgs a, int N, int L, cudaStream_t st, int list_words_
     const bool two = L > 16;
     const void* fn = lists == 2 ? (const void*)scl_kernel<false, 16>
                                 : (two ? (const void*)scl_kernel<true, 32> : (const void*)scl_kernel<false, 32>);
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e = raise_smem_limit(fn, smem);
     if (e != cudaSuccess) return e;
     int per_sm = 0;
     e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fn, W * 32, smem);

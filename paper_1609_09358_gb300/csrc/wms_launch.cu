@@ -17,11 +17,8 @@ static cudaError_t wms_launch_t(bool backward, const WMSArgs& a, cudaStream_t st
     const size_t smem = words * sizeof(float);
     static_assert((size_t)F * wms_slot_floats<P>() * sizeof(float) <= 48 * 1024 || LOGN == 11, "default limit");
     if (backward) {
-        if (smem > 48 * 1024) {
-            const cudaError_t e = cudaFuncSetAttribute((const void*)wms_backward_kernel<P, TH, CB>,
-                                                       cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            if (e != cudaSuccess) return e;
-        }
+        const cudaError_t e = raise_smem_limit((const void*)wms_backward_kernel<P, TH, CB>, smem);
+        if (e != cudaSuccess) return e;
         wms_backward_kernel<P, TH, CB><<<grid, TH, smem, st>>>(a);
     } else {
         wms_forward_kernel<P, TH, CF><<<grid, TH, smem, st>>>(a);
