@@ -433,6 +433,34 @@ struct BPKernelPlan<12, 0, 0, 1> {
     static constexpr int F = 1;
 };
 
+// Frame start and end of a kernel (FPT as above; SYNP as bp_run_group; QUEUE: the mixed kernel).  `tables`:
+// the code tables of a thread's consecutive nodes come in vectors and its decided bits are packed before
+// they go to shared memory; `llr_u`: LLR(u) leaves in 16-byte vectors; false: node by node.  Both are off
+// the iterations' path, but they change which registers the compiler keeps there.  The vector forms are
+// as fast or faster (mixed half2 by 8%, learned by 1 to 2.5%), but for the kernels named here, where they
+// cost spills or instructions in the loop.  Measured, node by node / vectors, BP of 40e6 / N / 2 frames,
+// i_max = 200 at 1.0 dB, in us: half2 N = 128 1968 / 1987, N = 1024 4402 / 4531 (4.9% with CRCs above 16
+// bits), N = 4096 by the LLR(u) store alone 7211 / 7434 (CRCs of at most 16 bits; 1.1% the other way above);
+// learned half2 past its learned iterations, N = 2048: 6.2%; FP32 N = 128 with CRCs above 16 bits 1.0%,
+// N = 2048 0.5%; re-encoding N = 4096 2889 / 2972 (1.5 dB), with the exact g N = 2048 0.9%.
+struct BPEnds {
+    bool tables, llr_u;
+};
+template <int LOGN, int WEIGHTED, int VAR, int FPT, bool SYNP, bool QUEUE>
+__host__ __device__ constexpr BPEnds bp_ends()
+{
+    if (QUEUE) return {true, true};
+    if (FPT == 2) {
+        if (WEIGHTED == 0 && (LOGN == 7 || LOGN == 10)) return {false, false};
+        if (WEIGHTED == 0 && LOGN == 12) return {true, !SYNP};
+        if (WEIGHTED == 1 && LOGN == 11) return {false, false};
+    } else if (WEIGHTED == 0) {
+        if (VAR == 0 && (LOGN == 11 || (LOGN == 7 && !SYNP))) return {false, false};
+        if ((VAR == 2 && LOGN == 12) || (VAR == 3 && LOGN == 11)) return {false, false};
+    }
+    return {true, true};
+}
+
 template <class P, bool CYC = false>
 __host__ __device__ constexpr int bp_slot_words()
 {
@@ -485,6 +513,9 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     static_assert(P::xidx_l(0) % 2 == 0, "odd number of exchanges per iteration");
     constexpr bool EXACT = (VAR & 1) != 0, REENC = (VAR & 2) != 0;
     constexpr bool UNIT = WEIGHTED == 2, ALIGNED = UNIT && FPT == 2;
+    constexpr bool QUEUE = std::is_same<Src, QueueSource>::value;
+    constexpr bool TABLES = bp_ends<n, WEIGHTED, VAR, FPT, SYNP, QUEUE>().tables;
+    constexpr bool LLRU = bp_ends<n, WEIGHTED, VAR, FPT, SYNP, QUEUE>().llr_u;
     static_assert(VAR == 0 || (FPT == 1 && !WEIGHTED), "exact g and the re-encoding stop: FP32, unweighted");
     static_assert(!REENC || (T % 32 == 0 && (!SHARED_CTA || T == 32)), "re-encoding vote: whole warps, own barrier");
     // PE function: min-sum (one instruction) or exact; the exact value is clipped like every
@@ -599,7 +630,7 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     // group 0's window is bits 0..b-1: a thread's nodes are R consecutive ones, inside one word of the
     // frozen mask
     static_assert(P::win(0) == 0 && 32 % R == 0 && R % 4 == 0, "consecutive nodes in group 0");
-    {
+    if constexpr (TABLES) {
         const int j0 = P::node(0, t, 0);
         const uint32_t fz = C.frozen_bits[j0 >> 5] >> (j0 & 31);
 #pragma unroll
@@ -616,6 +647,19 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
         }
 #pragma unroll
         for (int k = 0; k < R; ++k) Rc[1][k] = (fz >> k) & 1u ? Mv : MT::splat(0.0f);
+    } else {
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const int j = P::node(0, t, k);
+            const uint32_t col = C.colsyn[j];
+            if constexpr (syn_nodes) {
+                if (!(k & 1))
+                    csyn[(k >> 2) * 2 * T + 2 * t + ((k >> 1) & 1)] = col | (C.colsyn[P::node(0, t, k + 1)] << 16);
+            } else {
+                csyn[k * T + t] = syn_packed ? (col | (col << 16)) : col;
+            }
+            Rc[1][k] = frozen_at(C.frozen_bits, j) ? Mv : MT::splat(0.0f);
+        }
     }
     {
         const float* y0 = fr[0] >= 0 ? row(fr[0]) : nullptr;
@@ -690,7 +734,7 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
         uint32_t* pb = pbits + h * (N / 32);
         for (int i = t; i < N / 32; i += T) pb[i] = 0u;
         group_sync<T, SHARED_CTA>(slot);
-        {
+        if constexpr (TABLES) {
             // the payload positions among a thread's consecutive nodes are consecutive too: its bits are
             // packed first and go into one word, or two
             const short4* pp = reinterpret_cast<const short4*>(C.paypos + P::node(0, t, 0));
@@ -711,6 +755,12 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                 if ((uint32_t)w) atomicOr(&pb[first >> 5], (uint32_t)w);
                 if (w >> 32) atomicOr(&pb[(first >> 5) + 1], (uint32_t)(w >> 32));
             }
+        } else {
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int pos = C.paypos[P::node(0, t, k)];
+                if (pos >= 0 && MT::neg(fadd(Lc[1][k], Rc[1][k]), h)) atomicOr(&pb[pos >> 5], 1u << (pos & 31));
+            }
         }
         group_sync<T, SHARED_CTA>(slot);
         // the packed payload has ceil(P/8) <= N/8 bytes; a wider output row (a mixed batch uses
@@ -728,18 +778,24 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
             }
         }
         if (a.llr_u) {
-            float* lu = a.llr_u + (size_t)frame * N + P::node(0, t, 0);
+            if constexpr (LLRU) {
+                float* lu = a.llr_u + (size_t)frame * N + P::node(0, t, 0);
 #pragma unroll
-            for (int k = 0; k < R; k += 4) {
-                float u[4];
+                for (int k = 0; k < R; k += 4) {
+                    float u[4];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) u[q] = MT::to_f(fadd(Lc[1][k + q], Rc[1][k + q]), h);
-                if (a.out16) {
-                    *reinterpret_cast<float4*>(lu + k) = make_float4(u[0], u[1], u[2], u[3]);
-                } else {
+                    for (int q = 0; q < 4; ++q) u[q] = MT::to_f(fadd(Lc[1][k + q], Rc[1][k + q]), h);
+                    if (a.out16) {
+                        *reinterpret_cast<float4*>(lu + k) = make_float4(u[0], u[1], u[2], u[3]);
+                    } else {
 #pragma unroll
-                    for (int q = 0; q < 4; ++q) lu[k + q] = u[q];
+                        for (int q = 0; q < 4; ++q) lu[k + q] = u[q];
+                    }
                 }
+            } else {
+#pragma unroll
+                for (int k = 0; k < R; ++k)
+                    a.llr_u[(size_t)frame * N + P::node(0, t, k)] = MT::to_f(fadd(Lc[1][k], Rc[1][k]), h);
             }
         }
         if (a.llr_x) {
