@@ -215,6 +215,7 @@ struct BPArgs {
     int frame0;                // index of the launch's first frame (frames frame0 .. frame0 + B - 1)
     int out16;                 // llr_u on a 16-byte boundary
     int* balance;              // CYC: iterations skipped less a sixteenth of those run, over the launch
+    int follows;               // launched to start as the CTAs of the kernel before it leave (see bp_kernel)
 };
 
 // Message traits: FP32 (one frame per thread) or half2 (two frames per thread).
@@ -574,9 +575,9 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     // with the look at the loop's start, where the state would be L[2..n]).  That pays where failing frames
     // repeat (2 dB and up) and not where they wander (11% repeat at 1.5 dB, fewer below), so a launch
     // keeps the balance of what it skips and ends early if it falls; launch_bp follows it with the
-    // plain kernel on the same counter.  BP and a list of one, 10^5 frames, i_max = 200, plain / both:
-    // 40.35 / 40.54 ms at 1.0 dB, 29.1 / 29.3 at 1.5, 11.7 / 11.2 at 2.0, 4.07 / 3.69 at 2.5,
-    // 2.27 / 2.14 at 3.0, 1.64 / 1.66 at 3.5.
+    // plain kernel on the same counter.  BP of 10^5 frames, i_max = 200, plain / both: 37.54 / 37.58 ms
+    // at 1.0 dB, 27.37 / 27.42 at 1.5, 11.19 / 10.65 at 2.0, 3.91 / 3.51 at 2.5, 2.10 / 1.99 at 3.0,
+    // 1.50 / 1.54 at 3.5.
     constexpr bool CYC = (VAR & 4) != 0;
     static_assert(!CYC || (VAR == 4 && T > 32 && std::is_same<Src, CounterSource>::value), "repeats: plain FP32 min-sum");
     uint32_t* pbits = synp + 4 * NW;                       // [2 frame][N/32]
@@ -1227,6 +1228,10 @@ constexpr int bp_min_ctas()
     return WEIGHTED != 0 || ((VAR & 1) && LOGN <= 10) ? BPConfig<LOGN>::MIN_CTAS_W : BPConfig<LOGN>::MIN_CTAS;
 }
 
+// The plain kernel of a length whose frames go through the repeat-finding kernel first
+template <int LOGN, class MSG, int WEIGHTED, int VAR>
+constexpr bool bp_has_cyc() { return LOGN == 10 && std::is_same<MSG, float>::value && WEIGHTED == 0 && VAR == 0; }
+
 // Per-length kernel: F frame groups per CTA; THREADS = F * T (passed explicitly: launch bounds
 // take no dependent member expression).
 template <int LOGN, class MSG, int WEIGHTED, int THREADS, bool SYNP = false, int VAR = 0>
@@ -1242,7 +1247,17 @@ __global__ void __launch_bounds__(THREADS, bp_min_ctas<LOGN, WEIGHTED, VAR>()) b
     constexpr int FPT = MsgTraits<MSG>::FPT;
     CounterSource src{a.next, a.B, (int)((blockIdx.x * F + slot) * FPT), FPT, a.frame0};
     constexpr int words = bp_slot_words<P, (VAR & 4) != 0>();
+    // The repeat-finding kernel and the plain one that follows it take frames from one counter, so the
+    // second need not wait for the first: its CTAs start as those of the first leave (programmatic
+    // dependent launch).  When the first hands the batch over, its last frames run beside the second's; in
+    // stream order those took one frame's max_iters iterations on a nearly idle chip, 0.2 ms (16 384 frames
+    // at 1.0 / 1.5 dB: BP 6.49 / 4.76 ms, now 6.30 / 4.60).  What comes after in the stream waits for the second kernel
+    // alone, so one of its CTAs waits for the end of the first (whose CTAs have all started by then and
+    // wait for nothing).
+    if constexpr ((VAR & 4) != 0) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     bp_run_group<P, MSG, WEIGHTED, false, CounterSource, SYNP, VAR>(a, *a.code, slot, t, smem + slot * words, src);
+    if constexpr (bp_has_cyc<LOGN, MSG, WEIGHTED, VAR>())
+        if (a.follows && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 }  // namespace polar

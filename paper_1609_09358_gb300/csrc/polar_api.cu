@@ -350,12 +350,14 @@ static int bp_message(int precision) { return precision & ~(POLAR_G_EXACT | POLA
 
 // From these iteration limits and batch sizes on the FP32 min-sum kernel that recognises repeating frames
 // goes first (N = 1024).  It needs about 25 iterations to find a repetition, so failing frames have to
-// run on well beyond that (at 50 every batch measured 2 to 6% slower); and where it gives up (see CYC in
-// bp_kernel.cuh) its last frames overlap nothing for up to max_iters iterations, 0.16 ms at 200, which
-// has to be little of the whole batch (37 frames, all resident at once: 352 -> 368 us with it).
+// run on well beyond that (at 50 every batch measured 2 to 6% slower), and its iterations are longer, which
+// weighs until it gives up (see CYC in bp_kernel.cuh): BP of 16 384 frames, i_max = 200, plain / both, in
+// ms: 6.28 / 6.30 at 1.0 dB, 4.56 / 4.60, 1.95 / 1.87, 0.78 / 0.70 at 2.5, 0.49 / 0.46, 0.37 / 0.35 at
+// 3.5; 37 frames at 1.5 dB, which cannot give up in time: hybrid 352 / 368 us.
 constexpr int kBPCycleIters = 150, kBPCycleFrames = 16384;
 
-static int launch_bp_kernel(const BPKernelInfo& k, BPArgs& a, int fpt, cudaStream_t stream)
+// follows: start as the CTAs of the launch before it leave (see bp_kernel)
+static int launch_bp_kernel(const BPKernelInfo& k, BPArgs& a, int fpt, cudaStream_t stream, bool follows)
 {
     POLAR_CUDA(raise_smem_limit(k.fn, k.smem));
     const int groups = (a.B + fpt - 1) / fpt, F = k.groups_per_cta;
@@ -367,8 +369,19 @@ static int launch_bp_kernel(const BPKernelInfo& k, BPArgs& a, int fpt, cudaStrea
         if (e != cudaSuccess) return cuda_fail(e, "bp occupancy");
         grid = std::min(grid, std::max(1, per_sm) * scl_sm_count());
     }
+    a.follows = follows;
     void* args[] = {&a};
-    const cudaError_t e = cudaLaunchKernel(k.fn, dim3(grid), dim3(k.threads), args, k.smem, stream);
+    cudaLaunchAttribute attr{};
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(k.threads);
+    cfg.dynamicSmemBytes = k.smem;
+    cfg.stream = stream;
+    cfg.attrs = &attr;
+    cfg.numAttrs = follows ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelExC(&cfg, k.fn, args);
     return e == cudaSuccess ? POLAR_OK : cuda_fail(e, "bp_kernel launch");
 }
 
@@ -421,8 +434,10 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
                      batch >= kBPCycleFrames;
     const BPKernelInfo first = cyc ? bp_kernel_info_fp32_cyc(n, code->crc_len <= 16) : BPKernelInfo{nullptr, 0, 0, 0};
     int rc = POLAR_OK;
-    if (first.fn) rc = launch_bp_kernel(first, a, fpt, stream);
-    return rc ? rc : launch_bp_kernel(k, a, fpt, stream);
+    if (first.fn) rc = launch_bp_kernel(first, a, fpt, stream, false);
+    // (not for the chunks of hybrid_decode_host, which overlap on two streams as it is: 30 011 frames at 2.5 dB
+    // took 1.69 to 1.74 ms without, 1.76 with the second kernels starting early)
+    return rc ? rc : launch_bp_kernel(k, a, fpt, stream, first.fn != nullptr && batch == B);
 }
 
 static int check_bp_args(const polar_code* code, const float* llr, int B, int max_iters, float llr_max,

@@ -1,0 +1,89 @@
+"""The repeat-finding BP kernel and the plain one behind it, at a signal where most failing frames are
+skipped ahead and at one where the first kernel hands the batch over to the second: recorded in a CUDA
+graph, launched from two streams at once, and chunk by chunk from host memory.  Bits, status and
+iteration counts equal the oracle's."""
+import numpy as np
+import pytest
+
+import oracle
+from tests import frames as fr
+
+torch = pytest.importorskip("torch")
+pytestmark = [pytest.mark.gpu,
+              pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
+
+from paper_1609_09358_gb300 import api, build  # noqa: E402
+
+CASES = pytest.mark.parametrize("ebn0,grid", [(1.5, 4.0), (0.5, 0.0)])
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _lib():
+    build.build()
+    api.load()
+
+
+def batch(ebn0, grid):
+    """(code, LLRs, oracle's results) of 24 000 frames, 120 different ones."""
+    ocode = fr.oracle_code(1024, 512, 16)
+    _, llr = fr.frames(ocode, ebn0, 120, seed=71)
+    if grid:  # values on a coarse grid: almost every failing frame ends in a short period
+        llr = (np.round(llr / grid) * grid).astype(np.float32)
+    ref = oracle.hybrid_decode(llr, ocode, 200, 20.0, 2, precision="f32")
+    want = [oracle.payload_of(ref["u_hat"], ocode), ref["status"], ref["iters"]]
+    return fr.api_code(ocode), np.tile(llr, (200, 1)), [np.concatenate([w] * 200) for w in want]
+
+
+def same(code, bits, status, iters, want):
+    return (np.array_equal(api.unpack_bits(bits.cpu().numpy(), code.P), want[0])
+            and np.array_equal(status.cpu().numpy(), want[1])
+            and np.array_equal(iters.cpu().numpy().astype(np.int32), want[2]))
+
+
+@CASES
+def test_captured_in_a_graph(ebn0, grid):
+    code, llr, want = batch(ebn0, grid)
+    x = torch.from_numpy(llr).cuda()
+    dec = api.Decoder(code, x.shape[0], 2)
+    dec.hybrid(x, 200, 20.0)
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        dec.hybrid(x, 200, 20.0)
+    for _ in range(3):
+        for out in (dec.bits, dec.status, dec.iters):
+            out.zero_()
+        g.replay()
+        torch.cuda.synchronize()
+        assert same(code, dec.bits, dec.status, dec.iters, want)
+
+
+def test_two_streams_at_once():
+    """The two signals' batches beside each other, each call's CA-SCL directly behind its BP."""
+    jobs = []
+    for ebn0, grid in ((1.5, 4.0), (0.5, 0.0)):
+        code, llr, want = batch(ebn0, grid)
+        x = torch.from_numpy(llr).cuda()
+        jobs.append((code, x, want, api.Decoder(code, x.shape[0], 2), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(3):
+        for _, x, _, dec, stream in jobs:
+            dec.hybrid(x, 200, 20.0, stream=stream)
+    torch.cuda.synchronize()
+    for code, _, want, dec, _ in jobs:
+        assert same(code, dec.bits, dec.status, dec.iters, want)
+
+
+@CASES
+def test_from_host_memory(ebn0, grid):
+    code, llr, want = batch(ebn0, grid)
+    B = llr.shape[0]
+    bits = torch.zeros((B, code.row_bytes), dtype=torch.uint8).pin_memory()
+    status = torch.zeros(B, dtype=torch.uint8).pin_memory()
+    iters = torch.zeros(B, dtype=torch.int16).pin_memory()
+    ws = torch.zeros(api.polar_workspace_bytes(code, B, 2, api.POLAR_OP_HYBRID_HOST), dtype=torch.uint8, device="cuda")
+    x = torch.from_numpy(llr).pin_memory()
+    for _ in range(2):
+        api.hybrid_decode_host(code, x, 200, 20.0, api.POLAR_FP32, None, 2, bits, status, iters, ws)
+        torch.cuda.synchronize()
+        assert same(code, bits, status, iters, want)
