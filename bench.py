@@ -339,7 +339,7 @@ def main():
     ops_per_frame_iter = 6 * n * N + K   # 6 ops per PE half-iteration (2 add, 2 g, 2 clip) + CRC
     lanes = 128 * (2 if prec == api.POLAR_FP16 else 1)
     peak_ops = sms * lanes * sm_max_mhz * 1e6
-    bp_avg_ms = bp_ms / max(bp_n, 1)
+    bp_avg_ms = bp_ms / a.steps  # BP of one step: one launch, or two where repeating frames are looked for
     # every step decodes the same frames: total algorithmic ops of the timed BP launches over their
     # summed device time (= ops per launch / average launch time when a step is one launch)
     achieved = ops_per_frame_iter * float(iters.sum()) * a.steps / (bp_ms * 1e-3)
@@ -974,7 +974,7 @@ def run_mixed(a, world, rank, local):
                        "payload_bits_per_step": P_total,
                        "cache": "inputs larger than L2 (%.0f MB of LLRs per step), no flush" % (llr.numel() * 4 / 1e6)},
             "fer": h["fer"], "ber": h["ber"], "fallback_rate": h["fallback_rate"], "avg_bp_iters": h["avg_bp_iters"],
-            "gpu_launches": 5 * steps, "roofline": h["roofline"], "clocks": h["clocks"],
+            "gpu_launches": 8 * steps, "roofline": h["roofline"], "clocks": h["clocks"],
             "fp32": {k: v for k, v in out["fp32"].items() if k != "clocks"},
             "fp16_detail": {k: h[k] for k in ("bp_ms", "scl_ms", "autotune")}}
     if rank == 0:

@@ -309,9 +309,10 @@ int hybrid_decode_scheduled(const polar_code* code, const float* llr, int32_t B,
                             void* workspace, size_t ws_bytes, void* stream);
 
 /* Kernel timing for measurement (not a step of the paper).  While enabled on the calling host
- * thread, every decoder call brackets its BP and SCL kernel launches with CUDA events on the
- * launch stream.  polar_profile_read waits for the recorded events, returns the summed device
- * time in milliseconds and the launch count of each kernel kind, and clears the record. */
+ * thread, every decoder call brackets its BP and its SCL kernels with CUDA events on the launch
+ * stream (BP may be two kernels, one bracket).  polar_profile_read waits for the recorded events,
+ * returns the summed device time in milliseconds and the number of kernels launched of each kind,
+ * and clears the record. */
 int polar_profile_enable(int32_t on);
 int polar_profile_read(double* bp_ms, int32_t* bp_launches, double* scl_ms, int32_t* scl_launches);
 

@@ -282,6 +282,7 @@ static int aux_stream(int which, cudaStream_t* out)
 // ---------------------------------------------------------------------------- kernel timing
 struct ProfRecord {
     int kind;  // 0 BP, 1 SCL
+    int launches;
     cudaEvent_t start, stop;
 };
 struct ProfState {
@@ -310,9 +311,10 @@ static cudaEvent_t prof_event()
     return e;
 }
 
-// Brackets one kernel launch with events when timing is enabled.
+// Brackets the kernel launches of one decoding step with events when timing is enabled.
 struct ProfScope {
     int kind;
+    int launches = 1;
     cudaStream_t st;
     cudaEvent_t start = nullptr;
     ProfScope(int k, cudaStream_t s) : kind(k), st(s)
@@ -332,7 +334,7 @@ struct ProfScope {
         cudaEvent_t stop = prof_event();
         const cudaError_t rc = stop ? cudaEventRecord(stop, st) : cudaErrorUnknown;
         if (rc == cudaSuccess) {
-            g_prof.recs.push_back({kind, start, stop});
+            g_prof.recs.push_back({kind, launches, start, stop});
         } else {
             if (stop && g_prof.err == cudaSuccess) g_prof.err = rc;
             g_prof.pool.push_back(start);
@@ -434,7 +436,10 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
                      batch >= kBPCycleFrames;
     const BPKernelInfo first = cyc ? bp_kernel_info_fp32_cyc(n, code->crc_len <= 16) : BPKernelInfo{nullptr, 0, 0, 0};
     int rc = POLAR_OK;
-    if (first.fn) rc = launch_bp_kernel(first, a, fpt, stream, false);
+    if (first.fn) {
+        prof.launches = 2;
+        rc = launch_bp_kernel(first, a, fpt, stream, false);
+    }
     // (not for the chunks of hybrid_decode_host, which overlap on two streams as it is: 30 011 frames at 2.5 dB
     // took 1.69 to 1.74 ms without, 1.76 with the second kernels starting early)
     return rc ? rc : launch_bp_kernel(k, a, fpt, stream, first.fn != nullptr && batch == B);
@@ -1329,7 +1334,7 @@ int polar_profile_read(double* bp_ms, int32_t* bp_launches, double* scl_ms, int3
         if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, r.start, r.stop);
         if (e != cudaSuccess && rc == POLAR_OK) rc = cuda_fail(e, "polar_profile_read");
         t[r.kind] += ms;
-        cnt[r.kind] += 1;
+        cnt[r.kind] += r.launches;
         g_prof.pool.push_back(r.start);
         g_prof.pool.push_back(r.stop);
     }

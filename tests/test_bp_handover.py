@@ -87,3 +87,18 @@ def test_from_host_memory(ebn0, grid):
         api.hybrid_decode_host(code, x, 200, 20.0, api.POLAR_FP32, None, 2, bits, status, iters, ws)
         torch.cuda.synchronize()
         assert same(code, bits, status, iters, want)
+
+
+def test_profile_counts_both_kernels():
+    code, llr, _ = batch(1.5, 4.0)
+    x = torch.from_numpy(llr).cuda()
+    dec = api.Decoder(code, x.shape[0], 2)
+    counts = []
+    for imax in (50, 200):  # the plain kernel alone, both
+        api.polar_profile_enable(True)
+        dec.hybrid(x, imax, 20.0)
+        api.polar_profile_enable(False)
+        bp_ms, bp, scl_ms, scl = api.polar_profile_read()
+        assert bp_ms > 0 and scl_ms > 0 and scl == 1
+        counts.append(bp)
+    assert counts == [1, 2]
