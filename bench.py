@@ -321,6 +321,9 @@ def main():
         time.sleep(0.3)
     clocks = clk.summary(t_start, t_end)
     bp_ms, bp_n, scl_ms, scl_n = api.polar_profile_read()
+    # iterations that a step's BP ran: whole periods of frames whose messages repeat are counted, not run
+    reported = float(iters.sum())
+    ran = reported - api.polar_hybrid_skipped_iterations(dec.workspace)[0]
     ms = e0.elapsed_time(e1)
     if dist:
         dist.barrier()
@@ -340,9 +343,9 @@ def main():
     lanes = 128 * (2 if prec == api.POLAR_FP16 else 1)
     peak_ops = sms * lanes * sm_max_mhz * 1e6
     bp_avg_ms = bp_ms / a.steps  # BP of one step: one launch, or two where repeating frames are looked for
-    # every step decodes the same frames: total algorithmic ops of the timed BP launches over their
-    # summed device time (= ops per launch / average launch time when a step is one launch)
-    achieved = ops_per_frame_iter * float(iters.sum()) * a.steps / (bp_ms * 1e-3)
+    # every step decodes the same frames: total algorithmic ops of the iterations run in the timed BP
+    # launches over their summed device time
+    achieved = ops_per_frame_iter * ran * a.steps / (bp_ms * 1e-3)
     traffic, pipes = None, None
     ptag = "fp16" if prec == api.POLAR_FP16 else "fp32"
     tfile = os.path.join(ROOT, "profiles", "ncu_traffic.txt")
@@ -368,8 +371,9 @@ def main():
     ops10 = 10 * n * N + K
     roofline = {"bound": "alu", "achieved": achieved / 1e12, "peak": peak_ops / 1e12, "unit": "Top/s",
                 "frac": achieved / peak_ops, "traffic": traffic, "kernel": "bp_kernel",
-                "iterations": "as reported; whole periods of repeating frames are skipped, so achieved "
-                              "counts operations that were not run",
+                "iterations_run_per_frame": ran / B, "reported_rate": achieved / 1e12 * reported / ran,
+                "reported_rate_basis": "Top/s that the reported iteration counts would take: they include the "
+                                       "periods of repeating frames that are skipped",
                 "ops_per_frame_iter": ops_per_frame_iter, "bp_avg_ms": bp_avg_ms,
                 "peak_basis": "%d SMs x %d lanes x %.0f MHz (sm_max_mhz of MEASURED_PEAKS.json); 6 ops per PE "
                               "half-iteration = 3 comparison-pipe instructions at half rate" % (sms, lanes, sm_max_mhz),

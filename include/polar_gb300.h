@@ -382,6 +382,12 @@ size_t polar_workspace_bytes(const polar_code* code, int32_t B, int32_t L, int32
  * (host) after synchronising `stream`. */
 int polar_hybrid_fallback_count(const void* workspace, int32_t* out, void* stream);
 
+/* BP iterations that the last hybrid_decode on `workspace` counted without running them (whole
+ * periods of frames whose messages repeat; the reported iteration counts include them), copied to
+ * *out (host) after synchronising `stream`; *gave_up (host, may be NULL): 1 if too few frames
+ * repeated and the rest of the batch went without the search. */
+int polar_hybrid_skipped_iterations(const void* workspace, int64_t* out, int32_t* gave_up, void* stream);
+
 /* Message of the last failed call on this host thread ("" if none). */
 const char* polar_last_error(void);
 

@@ -83,6 +83,7 @@ SIGNATURES = {
                                           ctypes.POINTER(_i32)]),
     "polar_workspace_bytes": (_sz, [_CP, _i32, _i32, _i32]),
     "polar_hybrid_fallback_count": (ctypes.c_int, [_vp, ctypes.POINTER(_i32), _vp]),
+    "polar_hybrid_skipped_iterations": (ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int64), ctypes.POINTER(_i32), _vp]),
     "polar_last_error": (ctypes.c_char_p, []),
     "polar_pe_eval": (ctypes.c_int, [_i32, _vp, _vp, _vp, _i32, _vp]),
     "polar_pipe_rate_scratch_bytes": (_sz, []),
@@ -419,6 +420,15 @@ def polar_hybrid_fallback_count(workspace, stream=None) -> int:
     _check(load().polar_hybrid_fallback_count(_ptr(workspace), ctypes.byref(out), _stream(stream)),
            "polar_hybrid_fallback_count")
     return int(out.value)
+
+
+def polar_hybrid_skipped_iterations(workspace, stream=None):
+    """(iterations counted but not run, whether the search for them was given up) of the workspace's last
+    hybrid_decode."""
+    out, gave_up = ctypes.c_int64(0), _i32(0)
+    _check(load().polar_hybrid_skipped_iterations(_ptr(workspace), ctypes.byref(out), ctypes.byref(gave_up),
+                                                  _stream(stream)), "polar_hybrid_skipped_iterations")
+    return out.value, bool(gave_up.value)
 
 
 # ------------------------------------------------------------------------ convenience wrappers

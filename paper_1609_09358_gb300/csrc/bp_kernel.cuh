@@ -215,6 +215,7 @@ struct BPArgs {
     int frame0;                // index of the launch's first frame (frames frame0 .. frame0 + B - 1)
     int out16;                 // llr_u on a 16-byte boundary
     int* balance;              // CYC: iterations skipped less a sixteenth of those run, over the launch
+    unsigned long long* skipped;  // CYC: iterations skipped, over the launch
     int follows;               // launched to start as the CTAs of the kernel before it leave (see bp_kernel)
 };
 
@@ -1096,6 +1097,7 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                                 const int now = atomicAdd(a.balance, gain);
                                 if (now > (1 << 24)) atomicAdd(a.balance, -gain);  // far from the limit
                                 fetched[1] = now;
+                                if (skipped) atomicAdd(a.skipped, (unsigned long long)skipped);
                             }
                             group_sync<T, SHARED_CTA>(slot);
                             if (fetched[1] < kBPBalance) break;

@@ -195,6 +195,12 @@ struct ChunkHdr {
     int bp_balance;  // BPArgs::balance
 };
 static size_t hybrid_chunk_header_bytes(int) { return 256; }
+// The iterations that a hybrid call's BP skipped (BPArgs::skipped): in the first header, which every call
+// zeroes, behind WsHeader, on an 8-byte boundary wherever the workspace starts.
+static unsigned long long* hybrid_skipped(const void* base)
+{
+    return reinterpret_cast<unsigned long long*>(align_up(reinterpret_cast<uintptr_t>(base) + sizeof(WsHeader), 8));
+}
 
 // Device buffers of hybrid_decode_host: the whole batch's LLRs, bits, status and iterations, the
 // BP work counters of the chunks, and the hybrid workspace of the batch.
@@ -391,10 +397,11 @@ static int launch_bp(const DevCode* dcode, const polar_code* code, const float* 
                      float llr_max, int precision, const void* w, int w_iters, uint8_t* bits, uint8_t* status,
                      uint16_t* iters, float* llr_u, float* llr_x, int* fail_count, int* fail_list,
                      cudaStream_t stream, int* fail_total = nullptr, int* next = nullptr, int fixed_iters = 0,
-                     int frame0 = 0, int* balance = nullptr, int batch = 0)
+                     int frame0 = 0, int* balance = nullptr, unsigned long long* skipped = nullptr, int batch = 0)
 {
     BPArgs a{};
     a.balance = balance;
+    a.skipped = skipped;
     a.frame0 = frame0;
     a.fixed_iters = fixed_iters;
     a.fail_total = fail_total;
@@ -705,7 +712,8 @@ int hybrid_decode(const polar_code* code, const float* llr, int32_t B, int32_t m
     void* scratch = reinterpret_cast<char*>(list) + align_up(sizeof(int) * (size_t)B, 256);
     POLAR_CUDA(cudaMemsetAsync(base, 0, kHeaderBytes + sizeof(ChunkHdr), st));
     if ((rc = launch_bp(d, code, llr, B, max_iters, llr_max, precision, wms_scales, wms_iters, bits, status, iters,
-                        nullptr, nullptr, &hdr->fail_count, list, st, total, &hdr->bp_next, 0, 0, &hdr->bp_balance, B)))
+                        nullptr, nullptr, &hdr->fail_count, list, st, total, &hdr->bp_next, 0, 0, &hdr->bp_balance,
+                        hybrid_skipped(base), B)))
         return rc;
     return launch_scl(d, code, llr, B, L, bits, status, list, &hdr->fail_count, &hdr->scl_next, scratch, st);
 }
@@ -769,7 +777,7 @@ int hybrid_decode_host(const polar_code* code, const float* llr_host, int32_t B,
         POLAR_CUDA(cudaStreamWaitEvent(st, evc, 0));
         rc = launch_bp(d, code, llr_d, nb, max_iters, llr_max, precision, wms_scales, wms_iters, bits_d, status_d,
                        iters_d, nullptr, nullptr, &hdr->fail_count, list, st, total, counters + c, 0, b0,
-                       &hdr->bp_balance, B);
+                       &hdr->bp_balance, hybrid_skipped(wsb), B);
     }
     if (rc == POLAR_OK && (rc = event(&ev1)) == POLAR_OK) {
         POLAR_CUDA(cudaEventRecord(ev1, st1));
@@ -1370,6 +1378,20 @@ int polar_hybrid_fallback_count(const void* workspace, int32_t* out, void* strea
     POLAR_CUDA(cudaMemcpyAsync(&v, workspace, sizeof(int), cudaMemcpyDeviceToHost, st));
     POLAR_CUDA(cudaStreamSynchronize(st));
     *out = v;
+    return POLAR_OK;
+}
+
+int polar_hybrid_skipped_iterations(const void* workspace, int64_t* out, int32_t* gave_up, void* stream)
+{
+    if (!workspace || !out) return fail(POLAR_ERR_ARG, "NULL workspace/out");
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    unsigned long long v = 0;
+    ChunkHdr h{};
+    POLAR_CUDA(cudaMemcpyAsync(&v, hybrid_skipped(workspace), sizeof v, cudaMemcpyDeviceToHost, st));
+    POLAR_CUDA(cudaMemcpyAsync(&h, static_cast<const char*>(workspace) + kHeaderBytes, sizeof h, cudaMemcpyDeviceToHost, st));
+    POLAR_CUDA(cudaStreamSynchronize(st));
+    *out = (int64_t)v;
+    if (gave_up) *gave_up = h.bp_balance < kBPBalance;
     return POLAR_OK;
 }
 
