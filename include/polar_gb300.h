@@ -213,9 +213,9 @@ int wms_prepare(const polar_code* code, const float* w, int32_t wms_iters, int32
 
 /* Training of the learned weighted min-sum BP (the configurations' learned variant; not in the
  * paper).  wms_forward runs T iterations of the weighted BP of bp_decode (no early stop) and
- * writes LLR(u) = L_{.,1} + R_{.,1}, storing every message in the workspace: of the last
- * iteration into llr_u [B][N] (all_iters = 0), or of every iteration into llr_u [T][B][N]
- * (all_iters = 1, for a loss summed over iterations).  wms_backward, given dLoss/dLLR(u) in the
+ * writes LLR(u) = L_{.,1} + R_{.,1} of the last iteration into llr_u [B][N] (all_iters = 0), or of
+ * every iteration into llr_u [T][B][N] (all_iters = 1, for a loss summed over iterations), storing
+ * the messages of columns 2 to n, both sweeps, in the workspace.  wms_backward, given dLoss/dLLR(u) in the
  * same shape, writes dLoss/dw for w[T][2][n][N] (overwritten, summed over the batch) by a
  * hand-written reverse sweep through the stored messages (subgradients of min and clip).  Call
  * wms_backward after wms_forward with the same llr, w, all_iters and workspace.  llr, w, llr_u,

@@ -952,8 +952,9 @@ int wms_prepare(const polar_code* code, const float* w, int32_t wms_iters, int32
 size_t wms_workspace_bytes(const polar_code* code, int32_t B, int32_t T)
 {
     if (check_code(code) != POLAR_OK || B < 0 || T < 1 || code->N > POLAR_MAX_N_MIXED) return 0;
+    // WMSArgs::store, and room to start it on a 16-byte boundary
     const size_t n = (size_t)log2i(code->N), N = (size_t)code->N;
-    return (size_t)B * (2 * (size_t)T * n * N + 3 * (n + 2) * N) * sizeof(float);
+    return B == 0 ? 0 : (size_t)B * (size_t)T * 2 * (n - 1) * N * sizeof(float) + 16;
 }
 
 static int wms_common(const polar_code* code, const float* llr, int B, int T, float llr_max, const float* w,
@@ -975,8 +976,6 @@ static int wms_common(const polar_code* code, const float* llr, int B, int T, fl
     a.T = T;
     a.M = llr_max;
     a.w = w;
-    // the stored columns take 2 (n-1) N floats per frame and iteration, 16-byte aligned; the rest of
-    // the workspace is unused
     a.store = reinterpret_cast<float*>(align_up(reinterpret_cast<uintptr_t>(workspace), 16));
     a.code = d;
     a.w16 = (reinterpret_cast<uintptr_t>(w) & 15u) == 0;
