@@ -26,12 +26,12 @@ def _lib():
 
 
 def test_encoder_at_the_largest_batch():
-    """One byte of payload and 16 of codeword per frame; every row against the codeword of its byte."""
-    ocode = fr.oracle_code(128, 16, 8, design_rate=8 / 128)
-    pay = torch.arange(256, dtype=torch.uint8, device="cuda").repeat(2**23)[:BATCH].view(BATCH, 1)
+    """256 different payloads over and over; every row against its payload's codeword."""
+    ocode = fr.oracle_code(128, 64, 8)
+    bits = inputs.payload_bits(5, 0, 256, ocode.P)
+    pay = torch.from_numpy(api.pack_bits(bits)).cuda().repeat(2**23, 1)[:BATCH]
     cw = torch.zeros((BATCH, 16), dtype=torch.uint8, device="cuda")
     api.polar_encode(fr.api_code(ocode), pay, cw)
-    bits = api.unpack_bits(np.arange(256, dtype=np.uint8).reshape(256, 1), 8)
     row = torch.from_numpy(api.pack_bits(oracle.encode_batch(bits, ocode))).cuda()
     for b in range(0, BATCH, 2**28):  # a multiple of 256 rows
         part = cw[b:b + 2**28]
