@@ -436,31 +436,33 @@ struct BPKernelPlan<12, 0, 0, 1> {
 };
 
 // Frame start and end of a kernel (FPT as above; SYNP as bp_run_group; QUEUE: the mixed kernel).  `tables`:
-// the code tables of a thread's consecutive nodes come in vectors and its decided bits are packed before
-// they go to shared memory; `llr_u`: LLR(u) leaves in 16-byte vectors; false: node by node.  Both are off
-// the iterations' path, but they change which registers the compiler keeps there.  The vector forms are
-// as fast or faster (mixed half2 by 8%, learned by 1 to 2.5%), but for the kernels named here, where they
-// cost spills or instructions in the loop.  Measured, node by node / vectors, BP of 40e6 / N / 2 frames,
-// i_max = 200 at 1.0 dB, in us: half2 N = 128 1968 / 1987, N = 1024 4402 / 4531 (4.9% with CRCs above 16
-// bits), N = 4096 by the LLR(u) store alone 7211 / 7434 (CRCs of at most 16 bits; 1.1% the other way above);
-// learned half2 past its learned iterations, N = 2048: 6.2%; FP32 N = 128 with CRCs above 16 bits 1.0%,
-// N = 2048 0.5%; re-encoding N = 4096 2889 / 2972 (1.5 dB), with the exact g N = 2048 0.9%.
+// the code tables of a thread's consecutive nodes come in vectors, otherwise node by node; `pack`: its
+// decided bits are packed before they go to shared memory (always with `tables`), otherwise one by one;
+// `llr_u`: LLR(u) leaves in 16-byte vectors, otherwise node by node.  All this is off the iterations' path,
+// but it changes which registers the compiler keeps there.  The vector forms are as fast or faster
+// (mixed half2 by 8%, learned by 1 to 2.5%), but for the kernels named here, where they cost spills or
+// instructions in the loop.  Measured, node by node / vectors, BP of 40e6 / N / 2 frames, i_max = 200 at
+// 1.0 dB, in us: half2 N = 128 1968 / 1987, N = 1024 4402 / 4531 (packed, node by node: 4395, and 1.7%
+// less than one by one at 2.5 dB; CRCs above 16 bits: vectors 4.9% slower, packed 1.2%), N = 4096 by the
+// LLR(u) store alone 7211 / 7434 (CRCs of at most 16 bits; 1.1% the other way above); learned half2 past
+// its learned iterations, N = 2048: 6.2%; FP32 N = 128 with CRCs above 16 bits 1.0%, N = 2048 0.5%;
+// re-encoding N = 4096 2889 / 2972 (1.5 dB), with the exact g N = 2048 0.9%.
 struct BPEnds {
-    bool tables, llr_u;
+    bool tables, pack, llr_u;
 };
 template <int LOGN, int WEIGHTED, int VAR, int FPT, bool SYNP, bool QUEUE>
 __host__ __device__ constexpr BPEnds bp_ends()
 {
-    if (QUEUE) return {true, true};
+    if (QUEUE) return {true, true, true};
     if (FPT == 2) {
-        if (WEIGHTED == 0 && (LOGN == 7 || LOGN == 10)) return {false, false};
-        if (WEIGHTED == 0 && LOGN == 12) return {true, !SYNP};
-        if (WEIGHTED == 1 && LOGN == 11) return {false, false};
+        if (WEIGHTED == 0 && (LOGN == 7 || LOGN == 10)) return {false, LOGN == 10 && SYNP, false};
+        if (WEIGHTED == 0 && LOGN == 12) return {true, true, !SYNP};
+        if (WEIGHTED == 1 && LOGN == 11) return {false, false, false};
     } else if (WEIGHTED == 0) {
-        if (VAR == 0 && (LOGN == 11 || (LOGN == 7 && !SYNP))) return {false, false};
-        if ((VAR == 2 && LOGN == 12) || (VAR == 3 && LOGN == 11)) return {false, false};
+        if (VAR == 0 && (LOGN == 11 || (LOGN == 7 && !SYNP))) return {false, false, false};
+        if ((VAR == 2 && LOGN == 12) || (VAR == 3 && LOGN == 11)) return {false, false, false};
     }
-    return {true, true};
+    return {true, true, true};
 }
 
 template <class P, bool CYC = false>
@@ -517,6 +519,7 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
     constexpr bool UNIT = WEIGHTED == 2, ALIGNED = UNIT && FPT == 2;
     constexpr bool QUEUE = std::is_same<Src, QueueSource>::value;
     constexpr bool TABLES = bp_ends<n, WEIGHTED, VAR, FPT, SYNP, QUEUE>().tables;
+    constexpr bool PACK = bp_ends<n, WEIGHTED, VAR, FPT, SYNP, QUEUE>().pack;
     constexpr bool LLRU = bp_ends<n, WEIGHTED, VAR, FPT, SYNP, QUEUE>().llr_u;
     static_assert(VAR == 0 || (FPT == 1 && !WEIGHTED), "exact g and the re-encoding stop: FP32, unweighted");
     static_assert(!REENC || (T % 32 == 0 && (!SHARED_CTA || T == 32)), "re-encoding vote: whole warps, own barrier");
@@ -736,9 +739,9 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
         uint32_t* pb = pbits + h * (N / 32);
         for (int i = t; i < N / 32; i += T) pb[i] = 0u;
         group_sync<T, SHARED_CTA>(slot);
+        // the payload positions among a thread's consecutive nodes are consecutive too: packed, its bits go
+        // into one word, or two
         if constexpr (TABLES) {
-            // the payload positions among a thread's consecutive nodes are consecutive too: its bits are
-            // packed first and go into one word, or two
             const short4* pp = reinterpret_cast<const short4*>(C.paypos + P::node(0, t, 0));
             uint32_t v = 0;
             int first = -1;
@@ -756,6 +759,21 @@ __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, 
                 const uint64_t w = (uint64_t)v << (first & 31);
                 if ((uint32_t)w) atomicOr(&pb[first >> 5], (uint32_t)w);
                 if (w >> 32) atomicOr(&pb[(first >> 5) + 1], (uint32_t)(w >> 32));
+            }
+        } else if constexpr (PACK) {
+            uint32_t v = 0;
+            int first = -1;
+#pragma unroll
+            for (int k = 0; k < R; ++k) {
+                const int pos = C.paypos[P::node(0, t, k)];
+                if (first < 0) first = pos;
+                if (pos >= 0 && MT::neg(fadd(Lc[1][k], Rc[1][k]), h)) v |= 1u << (pos - first);
+            }
+            if (v) {
+                // (in 32-bit words: with the 64-bit shift half of what packing gains here is lost)
+                const uint32_t lo = v << (first & 31), hi = __funnelshift_l(v, 0u, first & 31);
+                if (lo) atomicOr(&pb[first >> 5], lo);
+                if (hi) atomicOr(&pb[(first >> 5) + 1], hi);
             }
         } else {
 #pragma unroll
