@@ -18,7 +18,7 @@
  *         ahead of or behind the call;
  *       * one page-locked host array of per-chunk failure counts for hybrid_decode_scheduled
  *         (4 bytes per chunk, grown when a call needs more, kept until exit), under a lock;
- *       * per device and kernel, whether the kernel's shared-memory limit was raised;
+ *       * per device and kernel, the shared-memory limit the kernel was last raised to;
  *       * the mixed BP plan table set by polar_mixed_autotune / polar_mixed_set_plan;
  *       * per host thread, the last error message and the profiling records of polar_profile_*
  *         (CUDA events, pooled).

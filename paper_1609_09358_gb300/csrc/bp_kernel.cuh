@@ -501,8 +501,9 @@ __host__ __device__ constexpr int pe_k(int dd, int i) { return ((i & ~(dd - 1)) 
 // so the scaled term needs no clip) and, for half2, both frames of a register kept on the same
 // iteration (a frame that stops waits for its partner; the pair refills together), so that one
 // binary16 scale, duplicated in the register, scales both -- used when every iteration is a
-// learned one.  (Scales stored as ready (w, w) pairs instead measured slower: twice the bytes
-// read from L2 per frame pair and iteration, which is what bounds the weighted kernel.)
+// learned one.  (Scales stored as ready (w, w) pairs instead measured slower, with twice the bytes
+// read from L2 per frame pair and iteration.  The kernel is bound by instruction issue: 72%, like its
+// ALU pipe, L2 at 22%.)
 template <class P, class MSG, int WEIGHTED, bool SHARED_CTA, class Src, bool SYNP = false, int VAR = 0>
 __device__ __forceinline__ void bp_run_group(const BPArgs& a, const DevCode& C, int slot, int t, uint32_t* slot_smem,
                                              Src& src)

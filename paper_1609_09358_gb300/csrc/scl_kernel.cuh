@@ -146,8 +146,8 @@ inline int scl_sm_count()
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     return sms > 0 ? sms : 1;
 }
-// List width of a CA-SCL launch: two frames per warp (half-warp lists) for L <= 8 in the global
-// layout with a single code.
+// List width of a CA-SCL launch, mixed batches included: two frames per warp (half-warp lists) for
+// L <= 8 in the global layout.
 inline bool scl_two_lists(int L, bool all_smem) { return L <= 8 && !all_smem; }
 // global workspace of the SCL list arrays (one slot per resident list: up to kSclWarpsPerSM lists
 // per SM)

@@ -30,9 +30,9 @@
 // access).  What bounds both kernels is that stream (2 (n-1) N floats per frame and iteration written
 // once, read twice, the second time from L2) and, for the backward one, a float reduction in L2 per
 // weight, frame and iteration.
-// Measured (N = 1024, T = 20, 4096 frames): forward 1.22 ms, backward 2.48 ms, against 2.98 and 8.71
+// Measured (N = 1024, T = 20, 4096 frames): forward 1.21 ms, backward 2.45 ms, against 2.98 and 8.71
 // for kernels with one PE per thread, every message (backward: every adjoint too) in memory and a
-// barrier after every stage.  Without the reductions the backward one takes 2.16 ms; with two frames
+// barrier after every stage.  Without the reductions the backward one took 2.16 ms; with two frames
 // per thread (half the scale loads and reductions, 600 bytes of spills) it took 3.7.
 #pragma once
 
@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(THREADS, CTAS) wms_forward_kernel(const WMSArg
 #pragma unroll
         for (int k = 0; k < R; ++k) Lc[c][k] = 0.0f;
     // scales of the stage being computed and of the next one (loaded a stage ahead: with loads at
-    // their use the forward kernel took 1.20 ms, the backward one 3.5)
+    // their use the forward kernel took the same, the backward one 3.5 ms)
     float wv[R], wn[R];
     th.template row<0>(a.w, a.w16, wn);
     for (int it = 0; it < a.T; ++it) {
